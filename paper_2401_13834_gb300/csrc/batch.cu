@@ -328,7 +328,7 @@ int build_batch(tx_batch* B, int64_t budget) {
       B->launches.push_back(L);
     }
     std::map<std::pair<int, int>, std::vector<int>> by_box;
-    for (int b : filt) by_box[{box_class(B->plans[b]->nw), B->plans[b]->output}].push_back(b);
+    for (int b : filt) by_box[{box_class(B->plans[b]->nw, B->plans[b]->output), B->plans[b]->output}].push_back(b);
     for (auto& kv : by_box) {
       BatchLaunch L;
       L.kind = kBoxcar;
