@@ -710,12 +710,12 @@ def run_ours(args):
             phases[name] = entry
         dom = max(phase_ms, key=phase_ms.get)
         if plan.interm == "f32":
-            kernel_of = {"ingest": "k_norm_ingest", "stage1": "k_stage1_f32", "stage2": "k_stage2_f32",
+            kernel_of = {"ingest": "k_norm_ingest", "stage1": "k_stage1_f32", "stage2": "k_stage2_pipe32",
                          "stats": "k_stats_f32", "boxcar": "k_boxcar_f32"}
         else:
             kernel_of = {"ingest": "k_ingest_tf", "stage1": "k_stage1", "stage2": "k_stage2_pipe" if plan.tile_split2
                          and plan.group <= 16 and plan.interm in ("u16", "f16") else
-                         ("k_stage2_u16" if plan.interm in ("u16", "f16") else "k_stage2_i32"),
+                         ("k_stage2_u16" if plan.interm in ("u16", "f16") else "k_stage2_pipe32"),
                          "stats": "k_stats", "boxcar": "k_boxcar"}
         d = phases[dom]
         roof = {"bound": d["bound"], "achieved": d["achieved"], "peak": d["peak"], "unit": d["unit"],

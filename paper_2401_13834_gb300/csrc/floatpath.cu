@@ -8,20 +8,21 @@
 //   k_norm_ingest   x' = (float(x) - mu_c) * w_c into the beam's float32 circular buffer
 //                   behind the carried tail (which keeps its own block's normalisation)
 //   k_stage1_f32    P[k][s][t] = sum_{c in s} x'[c][t + d1[k][c]]  (FP32, channels in order)
-//   k_stage2_f32    D[d][t]    = sum_s P[k(d)][s][t + d2[d][s]]     (FP32, sub-bands in order),
-//                   with per-tile sums of D and D^2 in double
+//   k_stage2_pipe32 D[d][t]    = sum_s P[k(d)][s][t + d2[d][s]]     (FP32, sub-bands in order),
+//                   with per-tile sums of D and D^2 (stage2_pipe32.cuh)
 //   k_stats_f32     mu_d, sigma_d of D over [0, T) in double (block or running)
 //   k_boxcar_f32    compensated (TwoSum) prefix sums of D per tile as float (hi, lo) pairs,
 //                   window sums B_W = C[t + W] - C[t], S/N = (B_W - W mu_d) / (sigma_d sqrt W)
-// Every thread of the de-dispersion stages computes one output by reading its
-// operands through the L1/L2 caches; the float path trades the integer path's
-// packed sums for arithmetic on normalised data.
+// The float path trades the integer path's packed sums for arithmetic on
+// normalised data.
 #include <cuda_runtime.h>
 
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
 
+#include "device.cuh"
+#include "stage2_pipe32.cuh"
 #include "tx_internal.h"
 
 using namespace tx;
@@ -211,86 +212,6 @@ __global__ void __launch_bounds__(kThreads1) k_stage1_f32(const float* __restric
   }
 }
 
-// 4-byte global -> shared copy that completes asynchronously (cp.async)
-__device__ __forceinline__ void cp_async4f(float* smem, const float* gmem) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(static_cast<uint32_t>(__cvta_generic_to_shared(smem))),
-               "l"(gmem) : "memory");
-}
-
-// One block per (tile of 2 NW outputs, coarse group k), one warp per fine DM
-// of the group: sub-band chunks of SC rows of P (the tile plus the group's
-// delay spread) are staged in shared memory, two buffers deep (chunk c + 1's
-// copies are in flight while chunk c is summed), and each warp sums its DM's
-// shifted rows in sub-band order, V = 2 NW / 32 outputs per lane; then the
-// tile's sums of D and D^2 over t < T in double to part[d][tile].
-template <int NW>
-__global__ void __launch_bounds__(kStage2MaxGroup * 32) k_stage2_f32(const float* __restrict__ P, int64_t Pp,
-                                                                      const int32_t* __restrict__ e2, int ndm, int nsub,
-                                                                      int G, int SC, int SW, float* __restrict__ D,
-                                                                      int64_t Dp, int64_t Td, int64_t T,
-                                                                      double2* __restrict__ part, int ntile) {
-  extern __shared__ float Sf[];   // [2][SC][SW]
-  constexpr int V = 2 * NW / 32;
-  const int tile = blockIdx.x, k = blockIdx.y;
-  const int64_t t0 = (int64_t)tile * 2 * NW;
-  const int dfirst = k * G;
-  const int nd = min(G, ndm - dfirst);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nch = (nsub + SC - 1) / SC;
-  // chunk c into buffer c & 1 (the group's first DM's delay is each row's start)
-  auto stage = [&](int c) {
-    const int sb = c * SC, ns = min(SC, nsub - sb);
-    float* dst = Sf + (size_t)(c & 1) * SC * SW;
-    for (int ss = 0; ss < ns; ++ss) {
-      const int s = sb + ss;
-      const float* src = P + ((size_t)k * nsub + s) * Pp + t0 + __ldg(e2 + (size_t)dfirst * nsub + s);
-      for (int j = threadIdx.x; j < SW; j += blockDim.x) cp_async4f(dst + (size_t)ss * SW + j, src + j);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  float acc[V];
-#pragma unroll
-  for (int v = 0; v < V; ++v) acc[v] = 0.f;
-  stage(0);
-  for (int c = 0; c < nch; ++c) {
-    if (c + 1 < nch) {
-      stage(c + 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");   // chunk c has landed
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
-    __syncthreads();
-    const int sb = c * SC, ns = min(SC, nsub - sb);
-    const float* buf = Sf + (size_t)(c & 1) * SC * SW;
-    if (warp < nd) {
-      for (int ss = 0; ss < ns; ++ss) {
-        const int s = sb + ss;
-        const int o = __ldg(e2 + (size_t)(dfirst + warp) * nsub + s) - __ldg(e2 + (size_t)dfirst * nsub + s);
-        const float* rw = buf + (size_t)ss * SW + o + lane;
-#pragma unroll
-        for (int v = 0; v < V; ++v) acc[v] = __fadd_rn(acc[v], rw[32 * v]);
-      }
-    }
-    __syncthreads();   // every warp is done with buffer c & 1 before chunk c + 2 lands there
-  }
-  if (warp < nd) {
-    const int d = dfirst + warp;
-    double s1 = 0.0, s2 = 0.0;
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const int64_t t = t0 + lane + 32 * v;
-      if (t < Td) D[(size_t)d * Dp + t] = acc[v];
-      if (t < T) { s1 += (double)acc[v]; s2 += (double)acc[v] * (double)acc[v]; }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
-    if (lane == 0) part[(size_t)d * ntile + tile] = make_double2(s1, s2);
-  }
-}
-
 // mu_d = sum D / T, var_d = sum D^2 / T - mu_d^2 (at least 0), or their running
 // update; (mu_d, sigma_d) to ms[d].
 __global__ void k_stats_f32(const double2* __restrict__ part, int ntile, int ndm, int64_t T, int running, double lam,
@@ -476,6 +397,18 @@ int normalise_into(const tx_plan* p, const uint8_t* src, int64_t n, int64_t pitc
 
 }  // namespace
 
+int float_upload(const tx_plan* p) {
+  TX_CUDA(raise_smem_limit((const void*)pipe32_kernel<float>(p), pipe32_smem(p)));
+  return TX_OK;
+}
+
+int float_wait_timeouts(int64_t* n) {
+  int v = 0;
+  TX_CUDA(cudaMemcpyFromSymbol(&v, g_tx_wait_timeouts, sizeof(int)));
+  *n = v;
+  return TX_OK;
+}
+
 int float_prime(const tx_plan* p, tx_beam* b, const uint8_t* d_tail, void* stream) {
   // the primed tail is normalised by its own statistics, as a block of L samples
   if (p->L <= 0) return TX_OK;
@@ -533,25 +466,11 @@ int float_execute(const tx_plan* p, tx_beam* b, const uint8_t* d_block, void* d_
   if ((rc = mark(2))) return rc;
 
   // stage 2 with per-tile sums
-  const dim3 g2((unsigned)p->ntile2, (unsigned)p->nk);
-  const int threads2 = std::min(p->group, kStage2MaxGroup) * 32;
-  // two buffers of chunks, about 56 KB in all, so that four blocks share an SM
-  const int sc2 = std::max(1, std::min(p->nsub_chunk2, (28 * 1024) / (p->sw2_i32 * (int)sizeof(float))));
-  const int smem2 = 2 * sc2 * p->sw2_i32 * (int)sizeof(float);
-#define TX_F2(NW)                                                                                                 \
-  do {                                                                                                            \
-    TX_CUDA(cudaFuncSetAttribute((const void*)k_stage2_f32<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem2)); \
-    k_stage2_f32<NW><<<g2, threads2, smem2, st>>>(P, p->Pp, p->dev.e2, p->ndm, p->nsub, p->group, sc2,            \
-                                                  p->sw2_i32, D, Dp, p->Td, p->T, part, p->ntile2);              \
-  } while (0)
-  if (p->nw2 == 512) TX_F2(512);
-  else TX_F2(256);
-#undef TX_F2
-  TX_CUDA(cudaGetLastError());
+  TX_CUDA(launch_stage2_pipe32<float>(p, P, D, Dp, part, b->run, st));
   if ((rc = mark(3))) return rc;
 
   if (!series) {
-    k_stats_f32<<<(p->ndm + 127) / 128, 128, 0, st>>>(part, p->ntile2f, p->ndm, p->T, p->stats == TX_STATS_RUNNING,
+    k_stats_f32<<<(p->ndm + 127) / 128, 128, 0, st>>>(part, p->ntile2 * p->split32, p->ndm, p->T, p->stats == TX_STATS_RUNNING,
                                                       p->lambda, b->run, ms);
     TX_CUDA(cudaGetLastError());
     if ((rc = mark(4))) return rc;

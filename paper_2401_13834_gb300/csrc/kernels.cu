@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "kernels.cuh"
+#include "stage2_pipe32.cuh"
 #include "tx_internal.h"
 
 using namespace tx;
@@ -42,7 +43,7 @@ bool is16(const tx_plan* p) { return p->interm == TX_INTERM_U16 || p->interm == 
 int stage2_smem(const tx_plan* p) {
   if (p->pipe2) return (int)stage2_pipe_smem(p->nsub_chunk2, p->sww2);
   if (is16(p)) return stage2_u16_smem_for(p->nsub_chunk2 * p->sww2, p->nsub_chunk2, p->e2w2);
-  return p->nsub_chunk2 * p->sw2_i32 * 4;
+  return pipe32_smem(p);
 }
 
 int box_smem(const tx_plan* p) { return box_smem_for(p->box_tile, p->wmax); }
@@ -100,10 +101,10 @@ int do_upload(tx_plan* p) {
       default: rc = set_stage2_attr<256, 32, 1>(s2); break;
     }
     if (rc) return rc;
-  } else if (p->nw2 == 512) {
-    TX_CUDA(raise_smem_limit((const void*)k_stage2_i32<512>, s2));
-  } else {
-    TX_CUDA(raise_smem_limit((const void*)k_stage2_i32<256>, s2));
+  } else if (p->interm == TX_INTERM_I32) {
+    TX_CUDA(raise_smem_limit((const void*)pipe32_kernel<int32_t>(p), s2));
+  } else if ((rc = float_upload(p))) {
+    return rc;
   }
   if (p->output != TX_OUT_SERIES) {
     const BoxKernel<OneBeam> bk = box_kernel<OneBeam>(p->nw, p->output);
@@ -481,12 +482,7 @@ int execute_impl(const tx_plan* p, tx_beam* b, const uint8_t* d_block, void* d_o
       }
 #undef TX_S2
     } else {
-      const int threads = std::min(p->group, kStage2MaxGroup) * 32;
-      dim3 grid((unsigned)p->ntile2, (unsigned)p->nk);
-      const int32_t* P = static_cast<const int32_t*>(a.P);
-      launch_pdl(p->nw2 == 512 ? k_stage2_i32<512> : k_stage2_i32<256>, grid, threads, (size_t)stage2_smem(p), st, P,
-                 p->Pp, p->dev.e2, p->ndm, p->nsub, p->group, p->nsub_chunk2, p->sw2_i32, a.D, a.Dp, p->Td, p->T,
-                 a.part, p->ntile2);
+      TX_CUDA(launch_stage2_pipe32<int32_t>(p, static_cast<const int32_t*>(a.P), a.D, a.Dp, a.part, a.run, st));
     }
     TX_CUDA(cudaGetLastError());
   }
@@ -616,10 +612,11 @@ int32_t tx_wait_timeouts(int64_t* count) {
   if (!count) { set_error("null argument"); return TX_ERR_INVALID_ARG; }
   int v = 0;
   TX_CUDA(cudaMemcpyFromSymbol(&v, g_tx_wait_timeouts, sizeof(int)));
-  int64_t nb = 0;
-  const int rc = batch_wait_timeouts(&nb);
+  int64_t nb = 0, nf = 0;
+  int rc = batch_wait_timeouts(&nb);
+  if (rc == TX_OK) rc = float_wait_timeouts(&nf);
   if (rc) return rc;
-  *count = v + nb;
+  *count = v + nb + nf;
   return TX_OK;
 }
 

@@ -31,10 +31,9 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
-#include <map>
-#include <mutex>
 #include <utility>
 
+#include "device.cuh"
 #include "tx_internal.h"
 
 namespace {
@@ -136,75 +135,6 @@ __device__ __forceinline__ void madd(uint32_t& acc, uint32_t a, uint32_t one) {
 __device__ __forceinline__ void madd_hi16(uint32_t& acc, uint32_t a) {
   asm("mad.hi.u32 %0, %1, 65536, %0;" : "+r"(acc) : "r"(a));
 }
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(smem)), "l"(gmem));
-}
-__device__ __forceinline__ void cp_async4(void* smem, const void* gmem) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(smem)), "l"(gmem));
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;"); }
-
-// Bulk (TMA) copies into shared memory, completed on an mbarrier: the
-// issuing side announces the byte count (expect_tx, one arrival) and each
-// copy completes its bytes on the barrier; waiting threads poll the phase.
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void fence_mbar_init() { asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory"); }
-// orders this CTA's earlier generic-proxy accesses of shared memory before later bulk copies into it
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.expect_tx.shared.b64 st, [%0], %1;\n\t}"
-               ::"r"(smem_addr(bar)), "r"(bytes) : "memory");
-}
-// global -> shared, `bytes` a multiple of 16, both addresses 16-byte aligned
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-               ::"r"(smem_addr(dst)), "l"(src), "r"(bytes), "r"(smem_addr(bar)) : "memory");
-}
-// waits for phase `parity` of bar to complete, giving up after max_iter polls
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, uint32_t max_iter) {
-  for (uint32_t i = 0; i < max_iter; ++i) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(smem_addr(bar)), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
-constexpr uint32_t kMbarPolls = kWaitPolls;   // the full limit
-
-// Waits that gave up (a copy that never completed) in this translation
-// unit's kernels; a kernel that saw one returns early and its results are not
-// valid. Read by tx_wait_timeouts.
-__device__ int g_tx_wait_timeouts = 0;
-// Records a wait that gave up: in the counter above and in the beam's own
-// count, which marks the beam's state (tail, running statistics) and every
-// later result as not valid until the beam is reset or imported.
-template <typename A>
-__device__ __forceinline__ void record_give_up(const A& a) {
-  atomicAdd(&g_tx_wait_timeouts, 1);
-  if (a.run) atomicAdd(reinterpret_cast<int32_t*>(a.run + 2 * (size_t)a.ndm), 1);
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// Programmatic dependent launch: a kernel launched with programmatic stream
-// serialization may start while the kernel before it in the stream is still
-// finishing. Each kernel of the path waits (pdl_wait) before it touches
-// memory, so it runs on the completed results of everything before it; and
-// lets the next kernel start launching at once (pdl_trigger), so that the
-// next kernel's launch and block set-up overlap this one's tail. Both are
-// no-ops for a kernel launched without the attribute.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // ---------------------------------------------------------------------------
 // ingest (Sec. 2.3 data flow)
@@ -1166,28 +1096,6 @@ k_stage2_u16(const Src src, const int32_t* __restrict__ uoff, const int32_t* __r
 constexpr int kPipeStages = kPipeStages2;
 constexpr int kPipeProc = kPipeProd2 - 1;   // processing warps (the other producer warp issues)
 
-__device__ __forceinline__ bool mbar_try(uint64_t* bar, uint32_t parity) {
-  uint32_t done;
-  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-               : "=r"(done)
-               : "r"(smem_addr(bar)), "r"(parity)
-               : "memory");
-  return done != 0u;
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared.b64 st, [%0];\n\t}" ::"r"(smem_addr(bar)) : "memory");
-}
-// Bounded wait that also gives up as soon as another thread of the block has
-// raised the abort flag.
-__device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parity, uint32_t polls,
-                                                   const volatile int* abort) {
-  for (uint32_t i = 0; i < polls; ++i) {
-    if (mbar_try(bar, parity)) return true;
-    if (*abort) return false;
-  }
-  return false;
-}
-
 // The walk of one role over the block's chunks: unit, chunk within the unit,
 // tile, which member's arguments apply, and the few of them every chunk uses
 // (read once per unit: a batched launch finds them in constant memory at a
@@ -1490,61 +1398,6 @@ k_stage2_pipe(const Src src, const int32_t* __restrict__ uoff, const int32_t* __
       }
     }
     if (!cc.next(src, uoff, umem, nmem, nunits)) break;
-  }
-}
-
-// Stage 2 from int32 intermediates (plain layout, one output per load); one
-// block per (tile of 2 NW outputs, coarse group), sub-band chunks in turn.
-template <int NW>
-__global__ void __launch_bounds__(kStage2MaxGroup * 32)
-k_stage2_i32(const int32_t* __restrict__ P, int64_t Pp, const int32_t* __restrict__ e2, int ndm, int nsub,
-             int G, int SC, int SW, int32_t* __restrict__ D, int64_t Dp, int64_t Td, int64_t T,
-             longlong2* __restrict__ part, int ntile) {
-  extern __shared__ __align__(16) uint32_t smem3[];
-  pdl_wait();
-  pdl_trigger();
-  constexpr int V = 2 * NW / 32;
-  const int tile = blockIdx.x, k = blockIdx.y;
-  const int64_t t0 = (int64_t)tile * 2 * NW;
-  const int dfirst = k * G;
-  const int nd = min(G, ndm - dfirst);
-  int32_t* S = reinterpret_cast<int32_t*>(smem3);
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int32_t acc[V];
-#pragma unroll
-  for (int v = 0; v < V; ++v) acc[v] = 0;
-  for (int sb = 0; sb < nsub; sb += SC) {
-    const int ns = min(SC, nsub - sb);
-    for (int i = threadIdx.x; i < ns * SW; i += blockDim.x) {
-      const int ss = i / SW, j = i - ss * SW;
-      const int s = sb + ss;
-      S[(size_t)ss * SW + j] = __ldg(P + ((size_t)k * nsub + s) * Pp + t0 + e2[(size_t)dfirst * nsub + s] + j);
-    }
-    __syncthreads();
-    if (warp < nd) {
-      for (int ss = 0; ss < ns; ++ss) {
-        const int s = sb + ss;
-        const int o = e2[(size_t)(dfirst + warp) * nsub + s] - e2[(size_t)dfirst * nsub + s];
-        const int32_t* rw = S + (size_t)ss * SW + o + lane;
-#pragma unroll
-        for (int v = 0; v < V; ++v) acc[v] += rw[32 * v];
-      }
-    }
-    __syncthreads();
-  }
-  if (warp < nd) {
-    const int d = dfirst + warp;
-    int32_t* drow = D + (size_t)d * Dp;
-    long long s1 = 0;
-    unsigned long long s2 = 0;
-#pragma unroll
-    for (int v = 0; v < V; ++v) {
-      const int64_t t = t0 + lane + 32 * v;
-      if (t < Td) drow[t] = acc[v];
-      if (t < T) { s1 += acc[v]; s2 += (unsigned long long)((long long)acc[v] * acc[v]); }
-    }
-    warp_sum_stats(s1, s2);
-    if (lane == 0) part[(size_t)d * ntile + tile] = make_longlong2(s1, (long long)s2);
   }
 }
 
@@ -2074,42 +1927,6 @@ __global__ void k_fill_run(double* run, int n) {
 // ---------------------------------------------------------------------------
 // host helpers shared by the single-beam and batched launchers
 // ---------------------------------------------------------------------------
-// Launches kernel k with programmatic stream serialization (see pdl_wait):
-// the launch and block set-up overlap the tail of the kernel before it.
-template <typename... KArgs, typename... Args>
-cudaError_t launch_pdl(void (*k)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args&&... args) {
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = grid;
-  cfg.blockDim = block;
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, std::forward<Args>(args)...);
-}
-
-// Raises kernel k's dynamic shared memory limit on the current device to at
-// least `bytes`, never lowering it: plans of different shapes share kernels,
-// and the limit one plan needs must survive another plan's set-up.
-inline cudaError_t raise_smem_limit(const void* k, int bytes) {
-  static std::mutex mu;
-  static std::map<std::pair<int, const void*>, int> lim;
-  int dev = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  std::lock_guard<std::mutex> g(mu);
-  const auto key = std::make_pair(dev, k);
-  const auto it = lim.find(key);
-  const int cur = it == lim.end() ? 48 * 1024 : it->second;  // the default limit
-  if (bytes <= cur) return cudaSuccess;
-  e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (e == cudaSuccess) lim[key] = bytes;
-  return e;
-}
-
 // two buffers of (4 pad words + tile + look-ahead, rounded to 16-byte chunks)
 inline int box_smem_for(int tile, int wmax) { return 2 * ((tile + wmax + 8 + 3) & ~3) * 4; }
 
@@ -2217,7 +2034,7 @@ inline BeamArgs make_args(const tx_plan* p, const tx_beam* b, const uint8_t* blo
   a.nsub = p->nsub;
   a.ndm = p->ndm;
   a.G = p->group;
-  a.split2 = p->pipe2 ? p->split2 : 1;
+  a.split2 = p->pipe2 ? p->split2 : p->interm == TX_INTERM_I32 ? p->split32 : 1;
   a.SC = p->nsub_chunk2;
   a.SWW = p->sww2;
   a.ntile2 = p->ntile2;

@@ -227,6 +227,20 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
     p->split2 = G * 4 <= cmax ? 4 : G * 2 <= cmax ? 2 : 1;
     p->nw2 = 512;
   }
+  const bool is32 = !is16;
+  if (is32) {
+    // 32-bit intermediates: tiles of 1024 outputs (512 for groups of more than
+    // 16 DMs, two per warp), halved where one sub-band's staged row would not
+    // fit; as many of three stages as fit; warps per DM as the 16-bit pipeline
+    p->tile32 = G > 16 ? 512 : 1024;
+    auto sw = [&](int tile) { return (int)round_up(tile + (int64_t)span2 + 8, 4); };
+    const int least = G > 16 ? 256 : 512;
+    while (p->tile32 > least && stage2_pipe32_smem(1, 1, sw(p->tile32), G) > kSmemMax - 1024) p->tile32 /= 2;
+    p->sw32 = sw(p->tile32);
+    for (p->nstage32 = 3; p->nstage32 > 1 && stage2_pipe32_smem(p->nstage32, 1, p->sw32, G) > kSmemMax - 1024;) --p->nstage32;
+    p->split32 = G > 14 ? 1 : G > 7 ? 2 : 4;
+    p->nw2 = p->tile32 / 2;
+  }
   const int64_t tt2 = 2 * (int64_t)p->nw2;
   p->ntile2 = (int32_t)((p->Td + tt2 - 1) / tt2);
   p->sww2 = (int32_t)round_up(p->nw2 + (span2 + 7 + 2) / 2 + 6, 4);
@@ -245,15 +259,17 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
     const int64_t per_sub = 3 * (int64_t)p->sww2 * 4 + (int64_t)kStage2MaxGroup * 4 + 8;
     p->nsub_chunk2 = (int32_t)std::min<int64_t>(nsub, (kSmemMax - 1024 - 8 * (int64_t)p->e2w2) / per_sub);
   } else {
-    p->sw2_i32 = (int32_t)(tt2 + span2 + 16);
-    const int64_t per_sub = (int64_t)p->sw2_i32 * 4 + (int64_t)kStage2MaxGroup * 4 + 8;
-    p->nsub_chunk2 = (int32_t)std::min<int64_t>(nsub, (kSmemMax - 1024) / per_sub);
+    int32_t sc = nsub;
+    while (sc > 1 && stage2_pipe32_smem(p->nstage32, sc, p->sw32, G) > kSmemMax - 1024) --sc;
+    p->nsub_chunk2 = stage2_pipe32_smem(p->nstage32, sc, p->sw32, G) <= kSmemMax - 1024 ? sc : 0;
+    // the spread taken: a row of the nominal tile (512 outputs for one warp per DM, else 1024) and its slack
+    if (((split == 1 ? 512 : 1024) + (int64_t)span2 + 16) * 4 + kStage2MaxGroup * 4 + 8 > kSmemMax - 1024) p->nsub_chunk2 = 0;
   }
   if (p->nsub_chunk2 < 1) { set_error("stage-2 delay spread within a DM group (%d samples) too large; use a smaller group", span2); return TX_ERR_UNSUPPORTED; }
-  if (p->pipe2) {
+  if (p->pipe2 || is32) {
     // offsets of every (fine DM, sub-band) from its sub-band's staged row start,
     // which is the tile start plus the group's first (smallest) delay rounded
-    // down to 8 elements; tiles start at multiples of 1024
+    // down to 8 elements; tiles start at multiples of the tile length
     const int SC = p->nsub_chunk2, SCq = (SC + 3) & ~3, nch = (nsub + SC - 1) / SC;
     p->tab2.assign((size_t)nk * nch * (G + 1) * SCq, 0);
     for (int k = 0; k < nk; ++k)
@@ -285,7 +301,6 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
     if (units >= kBoxMinUnits) { p->box_tile = f * kBoxTile; break; }
   }
   p->ntile3 = (int32_t)((p->T + p->box_tile - 1) / p->box_tile);
-  p->ntile2f = p->ntile2;   // the float path's stage 2 uses the same tiles (2 nw2 outputs)
 
   // ---- stage-1 work list ----------------------------------------------------
   // quarter length q1: the largest of 256/128/64/32 whose staged words, raw
@@ -397,7 +412,7 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
   int64_t off = 0;
   p->ws_P = off; off = round_up(off + (int64_t)nk * nsub * p->Pp * psz, 256);
   p->ws_D = off; off = round_up(off + (p->output == TX_OUT_SERIES ? 0 : (int64_t)ndm * p->Dp * 4), 256);
-  const int64_t parts = fpath ? (int64_t)p->ntile2f : (int64_t)p->ntile2 * (p->pipe2 ? p->split2 : 1);
+  const int64_t parts = (int64_t)p->ntile2 * (p->pipe2 ? p->split2 : is32 ? p->split32 : 1);
   p->ws_part = off; off = round_up(off + (int64_t)ndm * parts * 16, 256);
   // S/N constants per (DM, width); the float path keeps (mu, sigma) per DM in double
   p->ws_const = off; off = round_up(off + std::max<int64_t>((int64_t)ndm * p->nw * (int64_t)sizeof(SnrConst), fpath ? (int64_t)ndm * 16 : 0), 256);

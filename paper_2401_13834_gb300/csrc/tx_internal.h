@@ -48,6 +48,12 @@ constexpr int64_t stage2_pipe_smem(int sc, int sww) {
   return (int64_t)kPipeStages2 * (2 * (int64_t)sc * sww + (int64_t)(kPipeMaxGroup2 + 1) * ((sc + 3) & ~3)) * 4;
 }
 
+// shared-memory bytes of the 32-bit pipelined stage 2 for `nst` stages of `sc`
+// sub-bands of `sw` elements and the offset tables of groups of `group` DMs
+constexpr int64_t stage2_pipe32_smem(int nst, int sc, int sw, int group) {
+  return (int64_t)nst * ((int64_t)sc * sw + (int64_t)(group + 1) * ((sc + 3) & ~3)) * 4;
+}
+
 // ---- matched filter ---------------------------------------------------------
 constexpr int kBoxTile = 2048;         // outputs per boxcar sub-tile (a unit holds 1, 2 or 4)
 constexpr int64_t kBoxMinUnits = 152 * 4 * 8;   // units a plan keeps for a full GPU before lengthening them
@@ -135,12 +141,13 @@ struct tx_plan {
   int32_t pipe2 = 0;              // 16-bit stage 2 runs as the barrier-free pipeline (groups <= 16)
   int32_t ntile2 = 0;             // stage-2 tiles over the series
   int32_t sww2 = 0;               // stage-2 staged words per sub-band (uint16 path)
-  int32_t sw2_i32 = 0;            // stage-2 staged elements per sub-band (int32 path)
+  // 32-bit intermediates (int32, float32): tile of outputs, staged elements per
+  // sub-band, stages in flight and warps per fine DM of the pipelined stage 2
+  int32_t tile32 = 0, sw32 = 0, nstage32 = 0, split32 = 0;
   int32_t nsub_chunk2 = 0;        // sub-bands staged at once by stage 2
   int32_t e2w2 = 0;               // words of one stage-2 group's delays in shared memory (rounded to 4)
   int32_t box_tile = tx::kBoxTile;  // boxcar outputs per unit (a multiple of kBoxTile)
   int32_t ntile3 = 0;             // boxcar units per DM over [0, T)
-  int32_t ntile2f = 0;            // float path: stage-2 tiles over the series (those of ntile2)
   int32_t tile_f = 0, span_f = 0;  // float path: stage-1 item length and delay spread limit
   std::vector<tx::Stage1Item> items_f;  // float path stage-1 items (s, coarse DMs [kb, ke), times)
   std::vector<tx::Stage1Item> items1;
@@ -151,7 +158,7 @@ struct tx_plan {
   // its residue mod 16 (every block when T is a multiple of 16)
   std::vector<int32_t> tab1;
   int32_t tab1_phase = 0;
-  // pipelined stage 2, per (coarse group k, sub-band chunk): rows g < group of
+  // pipelined stage 2 (16 and 32 bits), per (coarse group k, sub-band chunk): rows g < group of
   // SCq = (nsub_chunk2 + 3) & ~3 words, word ss = the element offset of fine
   // DM kG + g's pairs in sub-band s = chunk * nsub_chunk2 + ss from the start
   // of that sub-band's staged row, then one row of those starts relative to
@@ -193,5 +200,9 @@ int tx_upload_plan(const tx_plan* plan);
 int float_execute(const tx_plan* p, tx_beam* b, const uint8_t* d_block, void* d_out, int64_t* d_ncand,
                   void* d_workspace, void* stream, void* const* ev);
 int float_prime(const tx_plan* p, tx_beam* b, const uint8_t* d_tail, void* stream);
+// Sets the shared memory limits of the float path's kernels for plan p.
+int float_upload(const tx_plan* p);
+// Waits given up by the float path's kernels on the current device (floatpath.cu).
+int float_wait_timeouts(int64_t* n);
 // Waits given up by the batched kernels on the current device (batch.cu).
 int batch_wait_timeouts(int64_t* n);
