@@ -397,8 +397,8 @@ int normalise_into(const tx_plan* p, const uint8_t* src, int64_t n, int64_t pitc
 
 }  // namespace
 
-int float_upload(const tx_plan* p) {
-  TX_CUDA(raise_smem_limit((const void*)pipe32_kernel<float>(p), pipe32_smem(p)));
+int float_upload(tx_plan* p) {
+  TX_CUDA(upload_stage2_pipe32<float>(p));
   return TX_OK;
 }
 

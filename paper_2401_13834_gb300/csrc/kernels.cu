@@ -102,7 +102,7 @@ int do_upload(tx_plan* p) {
     }
     if (rc) return rc;
   } else if (p->interm == TX_INTERM_I32) {
-    TX_CUDA(raise_smem_limit((const void*)pipe32_kernel<int32_t>(p), s2));
+    TX_CUDA(upload_stage2_pipe32<int32_t>(p));
   } else if ((rc = float_upload(p))) {
     return rc;
   }

@@ -259,8 +259,10 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
     const int64_t per_sub = 3 * (int64_t)p->sww2 * 4 + (int64_t)kStage2MaxGroup * 4 + 8;
     p->nsub_chunk2 = (int32_t)std::min<int64_t>(nsub, (kSmemMax - 1024 - 8 * (int64_t)p->e2w2) / per_sub);
   } else {
+    // groups of few DMs make small blocks: room for as many as bring 32 warps to an SM
+    const int blocks = std::max(1, 32 / (std::min(G, 16) * p->split32 + 1));
     int32_t sc = nsub;
-    while (sc > 1 && stage2_pipe32_smem(p->nstage32, sc, p->sw32, G) > kSmemMax - 1024) --sc;
+    while (sc > 1 && stage2_pipe32_smem(p->nstage32, sc, p->sw32, G) > kSmemMax / blocks - 1024) --sc;
     p->nsub_chunk2 = stage2_pipe32_smem(p->nstage32, sc, p->sw32, G) <= kSmemMax - 1024 ? sc : 0;
     // the spread taken: a row of the nominal tile (512 outputs for one warp per DM, else 1024) and its slack
     if (((split == 1 ? 512 : 1024) + (int64_t)span2 + 16) * 4 + kStage2MaxGroup * 4 + 8 > kSmemMax - 1024) p->nsub_chunk2 = 0;

@@ -91,7 +91,8 @@ struct TileSums<float> {
 // rows with 4-byte copies between block-wide barriers. Waits are bounded as
 // in k_stage2_pipe.
 template <typename E, int VW, int NDM>
-__global__ void __launch_bounds__(VW * NDM >= 32 ? 544 : 928, 1) k_stage2_pipe32(const Pipe32Args<E> a) {
+__global__ void __launch_bounds__(VW * NDM >= 32 ? 544 : 928, 1)
+k_stage2_pipe32(const Pipe32Args<E> a) {
   extern __shared__ __align__(16) uint8_t smem32[];
   pdl_wait();
   pdl_trigger();
@@ -242,6 +243,18 @@ Pipe32Kernel<E> pipe32_kernel(const tx_plan* p) {
   return pipe32_kernel<E>(p->tile32 / 32 / p->split32, p->group > 16 ? 2 : 1);
 }
 
+// Sets its shared memory limit and the blocks that share an SM: several for
+// groups of few DMs (937 DMs in groups of 2, 2 sub-bands, 17507 outputs: 110 us
+// with one block of 9 warps per SM, 33 us with the blocks that fit).
+template <typename E>
+cudaError_t upload_stage2_pipe32(tx_plan* p) {
+  const Pipe32Kernel<E> k = pipe32_kernel<E>(p);
+  cudaError_t e = raise_smem_limit((const void*)k, pipe32_smem(p));
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p->dev.s2_blocks_per_sm, k, pipe32_threads(p), pipe32_smem(p));
+  return e;
+}
+
 // Launches the 32-bit stage 2 of plan p.
 template <typename E>
 cudaError_t launch_stage2_pipe32(const tx_plan* p, const E* P, E* D, int64_t Dp, void* part, double* run, cudaStream_t st) {
@@ -265,7 +278,7 @@ cudaError_t launch_stage2_pipe32(const tx_plan* p, const E* P, E* D, int64_t Dp,
   a.nstage = p->nstage32;
   a.split = p->split32;
   a.polls = first_wait_polls();
-  const int grid = std::min(a.nunits, std::max(p->dev.num_sms, 1));
+  const int grid = std::min(a.nunits, std::max(p->dev.num_sms, 1) * std::max(p->dev.s2_blocks_per_sm, 1));
   return launch_pdl(pipe32_kernel<E>(p), dim3(grid), dim3(pipe32_threads(p)), (size_t)pipe32_smem(p), st, a);
 }
 

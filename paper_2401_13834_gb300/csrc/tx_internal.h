@@ -85,6 +85,7 @@ struct DevicePlan {
   int device = -1;
   int num_sms = 0;
   int box_blocks_per_sm = 1;     // resident boxcar blocks per SM (persistent grid)
+  int s2_blocks_per_sm = 1;      // resident blocks per SM of the 32-bit stage 2
   int32_t* d1 = nullptr;         // [nk][nchan]
   int32_t* abase = nullptr;      // [nk][nsub]
   int32_t* e2 = nullptr;         // [ndm][nsub]
@@ -201,7 +202,7 @@ int float_execute(const tx_plan* p, tx_beam* b, const uint8_t* d_block, void* d_
                   void* d_workspace, void* stream, void* const* ev);
 int float_prime(const tx_plan* p, tx_beam* b, const uint8_t* d_tail, void* stream);
 // Sets the shared memory limits of the float path's kernels for plan p.
-int float_upload(const tx_plan* p);
+int float_upload(tx_plan* p);
 // Waits given up by the float path's kernels on the current device (floatpath.cu).
 int float_wait_timeouts(int64_t* n);
 // Waits given up by the batched kernels on the current device (batch.cu).
