@@ -146,68 +146,202 @@ __global__ void __launch_bounds__(kThreads) k_norm_ingest(const uint8_t* __restr
 }
 
 // ---- de-dispersion ----------------------------------------------------------------
-// One block per item (sub-band s, coarse DMs [kb, ke), absolute times
-// [tau0, tau0 + tile)): every channel's window of x' (tile + spread samples
-// from buffer position start + tau0 + d1[kb][c], mod R) is staged in shared
-// memory once, then each warp sums coarse DMs of the item over the
-// sub-band's channels in order, P[k][s][tau0 + j - abase[k][s]] = sum_c
-// S[c][j + d1[k][c] - d1[kb][c]], VW = tile / 32 outputs per lane.
-constexpr int kThreads1 = 1024;   // stage 1: a warp per coarse DM of an item (up to 32)
+// Stage 1: P[k][s][t] = sum_{c in s} x'[c][t + d1[k][c]], channels one after the
+// other (the sum order, and so every bit of the result, is part of the path).
+// Bound: shared memory, 4 bytes per sample-add that needs its own load (7.1 ms
+// for the 69e9 sample-adds of a MeerKAT-L block at 39.1 TB/s). A warp sums
+// four consecutive coarse DMs, and where neighbours have the same delay in a
+// channel they add the same registers: a quarter of the loads of a MeerKAT-L
+// block go that way.
+//
+// Persistent blocks walk the items (unit u = blockIdx.x + i gridDim.x) in
+// chunks of up to 16 channels through kF1Stages stages, without block-wide
+// barriers: the last warp bulk-copies (TMA) a chunk's windows of the ring, one
+// per lane (two where a window wraps the ring's end), and its offset table
+// (mbarriers full / empty); the others keep their four coarse DMs' sums in
+// registers over an item's chunks, VW outputs per lane. Tiles of 512 outputs
+// make a warp's part 256 outputs, 8 independent loads in flight per coarse DM,
+// for up to 40 coarse DMs on 20 warps.
+// One block per item that staged all its channels, then summed, took 12.57
+// ms on that block; this takes 7.63 ms with shared memory and issue both 80%
+// busy (every load taken: 8.30; 30 warps, which spill: 12.5; predicated loads
+// instead of branches, which keep their shared-memory slots: 8.25). Waits are
+// bounded as in k_stage2_pipe.
+struct F1Args {
+  const float* ring;
+  const Stage1Item* items;
+  const int32_t* chunks;
+  const uint32_t* tab;
+  const int32_t* abase;    // [nk][nsub]
+  float* P;
+  double* run;             // the beam's running statistics, then its count of given-up waits
+  int64_t R, start, Pp;
+  int32_t m, nsub, ndm, nitems;
+  int32_t phase;           // which of a chunk's tables
+  uint32_t polls;
+};
 
+struct F1Shared {
+  uint64_t full[kF1Stages], empty[kF1Stages];
+  int abort_flag;
+};
+
+// One item's sums by one consumer warp; false when a wait gave up.
 template <int VW>
-__global__ void __launch_bounds__(kThreads1) k_stage1_f32(const float* __restrict__ ring, int64_t R, int64_t start,
-                                                          const Stage1Item* __restrict__ items,
-                                                          const int32_t* __restrict__ d1,
-                                                          const int32_t* __restrict__ abase, int nchan, int m, int nsub,
-                                                          int64_t Pp, int sw, float* __restrict__ P) {
-  extern __shared__ float S[];   // [m][sw]
-  const Stage1Item it = items[blockIdx.x];
-  constexpr int tile = 32 * VW;
-  const int n = tile + it.span;
-  const int c0 = it.s * m;
-  const int32_t* d1b = d1 + (size_t)it.kb * nchan + c0;
-  // the windows: channel c from buffer position p0_c = (start + tau0 + d1[kb][c]) mod R on
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  for (int c = warp; c < m; c += kThreads1 / 32) {
-    const int64_t p0 = (start + it.tau0 + d1b[c]) % R;
-    const float* src = ring + (int64_t)(c0 + c) * R;
-    for (int j = lane; j < n; j += 32) {
-      int64_t p = p0 + j;
-      if (p >= R) p -= R;
-      S[c * sw + j] = __ldg(src + p);
+__device__ __forceinline__ bool f1_consume(const F1Args& a, F1Shared& sh, const float* stages, const Stage1Item& it,
+                                           int warp, int lane, int& st, uint32_t& par) {
+  constexpr int PARTS = kF1Tile / 32 / VW;
+  const int quads = (it.ke - it.kb + kF1Quad - 1) / kF1Quad;
+  const bool busy = warp < quads * PARTS;
+  const int quad = warp / PARTS, j0 = (warp - quad * PARTS) * 32 * VW + lane;   // this lane's first output
+  const int k0 = it.kb + quad * kF1Quad;
+  float acc[kF1Quad][VW];
+#pragma unroll
+  for (int i = 0; i < kF1Quad; ++i)
+#pragma unroll
+    for (int v = 0; v < VW; ++v) acc[i][v] = 0.f;
+  for (int left = a.m; left > 0; left -= kF1Chan) {
+    const int nc = min(left, kF1Chan);
+    if (!mbar_wait_or_abort(&sh.full[st], par, a.polls, &sh.abort_flag)) return false;
+    if (busy) {
+      const float* r = stages + (size_t)st * kF1StageWords + j0;
+      const uint2* t = reinterpret_cast<const uint2*>(stages + (size_t)st * kF1StageWords + kF1Chan * kF1RawWords) +
+                       quad * kF1Chan;
+      auto channel = [&](uint2 o) {
+        float x[VW];
+        uint32_t at = 0u;
+#pragma unroll
+        for (int i = 0; i < kF1Quad; ++i) {
+          const uint32_t w = i < 2 ? o.x : o.y;
+          const uint32_t oi = (i & 1) ? w >> 16 : w & 0xFFFFu;
+          if (i == 0 || oi != at) {   // a delay of its own
+#pragma unroll
+            for (int v = 0; v < VW; ++v) x[v] = r[oi + 32 * v];
+          }
+          at = oi;
+#pragma unroll
+          for (int v = 0; v < VW; ++v) acc[i][v] = __fadd_rn(acc[i][v], x[v]);
+        }
+      };
+      int c = 0;
+      for (; c + 1 < nc; c += 2) {
+        const uint4 o = *reinterpret_cast<const uint4*>(t + c);
+        channel(make_uint2(o.x, o.y));
+        channel(make_uint2(o.z, o.w));
+      }
+      if (c < nc) channel(t[c]);
     }
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&sh.empty[st]);
+    if (++st == kF1Stages) { st = 0; par ^= 1u; }
   }
-  __syncthreads();
-  for (int kk = warp; kk < it.ke - it.kb; kk += kThreads1 / 32) {
-    const int k = it.kb + kk;
-    const int32_t* d1k = d1 + (size_t)k * nchan + c0;
-    float acc[VW];
 #pragma unroll
-    for (int v = 0; v < VW; ++v) acc[v] = 0.f;
-    if (m <= 64) {
-      // the DM's channel offsets held two per lane and broadcast by shuffles:
-      // no global load between a channel's shared-memory loads
-      const int oa = lane < m ? __ldg(d1k + lane) - __ldg(d1b + lane) : 0;
-      const int ob = lane + 32 < m ? __ldg(d1k + lane + 32) - __ldg(d1b + lane + 32) : 0;
-      for (int c = 0; c < m; ++c) {
-        const int o = __shfl_sync(0xffffffffu, c < 32 ? oa : ob, c & 31);
-        const float* row = S + c * sw + o + lane;
+  for (int i = 0; i < kF1Quad; ++i) {
+    if (!busy || k0 + i >= it.ke) continue;
+    const size_t row = (size_t)(k0 + i) * a.nsub + it.s;
+    const int64_t j = (int64_t)it.tau0 - __ldg(a.abase + row) + j0;
+    float* prow = a.P + row * a.Pp;
 #pragma unroll
-        for (int v = 0; v < VW; ++v) acc[v] = __fadd_rn(acc[v], row[32 * v]);
+    for (int v = 0; v < VW; ++v)
+      if (j + 32 * v >= 0 && j + 32 * v < a.Pp) prow[j + 32 * v] = acc[i][v];
+  }
+  return true;
+}
+
+constexpr int kF1Threads = (kF1Consumers + 1) * 32;
+
+__global__ void __launch_bounds__(kF1Threads, 1) k_stage1_f32(const F1Args a) {
+  extern __shared__ __align__(16) float smf[];
+  __shared__ __align__(8) F1Shared sh;
+  pdl_wait();
+  pdl_trigger();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if ((int)blockIdx.x >= a.nitems) return;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < kF1Stages; ++i) {
+      mbar_init(&sh.full[i], 1);
+      mbar_init(&sh.empty[i], kF1Consumers);
+    }
+    sh.abort_flag = 0;
+    fence_mbar_init();
+  }
+  __syncthreads();   // barriers initialised: the only block-wide barrier
+  volatile int* abort = &sh.abort_flag;
+  auto give_up = [&]() {
+    if (atomicExch(&sh.abort_flag, 1) == 0) record_give_up(a);
+  };
+  int st = 0;
+  uint32_t par = 0u;
+
+  if (warp == kF1Consumers) {
+    // --------------------------------------------------------- the issuing warp
+    // (a chunk's record, and an item's descriptor, are loaded one ahead: the
+    // copies never wait for a dependent global load)
+    int64_t q = 0;
+    Stage1Item it = a.items[blockIdx.x], nx = it;
+    int u = blockIdx.x, ch = 0;
+    int rec = __ldg(a.chunks + (size_t)it.tab * kF1Rec + lane);
+    while (true) {
+      if (ch == 0 && u + (int)gridDim.x < a.nitems) nx = a.items[u + gridDim.x];
+      const bool more = ch + 1 < it.pad1 || u + (int)gridDim.x < a.nitems;
+      const int nrec = ch + 1 < it.pad1 ? it.tab + ch + 1 : nx.tab;
+      int rn = 0;
+      if (more) rn = __ldg(a.chunks + (size_t)nrec * kF1Rec + lane);
+      const int words = (3 + kF1Tile + it.span + 3) & ~3;   // a window: misalignment, tile, spread
+      const int cn = __shfl_sync(0xffffffffu, rec, 0), tw = __shfl_sync(0xffffffffu, rec, 1);
+      const int to = __shfl_sync(0xffffffffu, rec, 2), dl = __shfl_sync(0xffffffffu, rec, 8 + (lane & 15));
+      const int c0 = cn >> 5, nc = cn & 31;
+      if (q >= kF1Stages && !mbar_wait_or_abort(&sh.empty[st], par ^ 1u, a.polls, abort)) {
+        give_up();
+        break;
       }
-    } else {
-      for (int c = 0; c < m; ++c) {
-        const float* row = S + c * sw + (__ldg(d1k + c) - __ldg(d1b + c)) + lane;
-#pragma unroll
-        for (int v = 0; v < VW; ++v) acc[v] = __fadd_rn(acc[v], row[32 * v]);
+      float* dst = smf + (size_t)st * kF1StageWords;
+      if (lane == 0) mbar_expect_tx(&sh.full[st], (uint32_t)(nc * words + tw) * 4u);
+      __syncwarp();
+      fence_proxy_async();
+      if (lane < nc) {
+        int64_t p = a.start + it.tau0 + dl;
+        while (p >= a.R) p -= a.R;
+        const int64_t pa = p & ~(int64_t)3;
+        const float* row = a.ring + (size_t)(c0 + lane) * a.R;
+        float* d = dst + lane * kF1RawWords;
+        const int first = (int)min((int64_t)words, a.R - pa);
+        bulk_g2s(d, row + pa, (uint32_t)first * 4u, &sh.full[st]);
+        if (first < words) bulk_g2s(d + first, row, (uint32_t)(words - first) * 4u, &sh.full[st]);
+      }
+      if (lane == 31)
+        bulk_g2s(dst + kF1Chan * kF1RawWords, a.tab + (size_t)to * 4 + (size_t)a.phase * tw, (uint32_t)tw * 4u,
+                 &sh.full[st]);
+      ++q;
+      if (++st == kF1Stages) { st = 0; par ^= 1u; }
+      if (!more) break;
+      rec = rn;
+      if (++ch == it.pad1) {
+        ch = 0;
+        u += gridDim.x;
+        it = nx;
       }
     }
-    const int64_t rel = (int64_t)it.tau0 - abase[(size_t)k * nsub + it.s];
-    float* prow = P + ((size_t)k * nsub + it.s) * Pp;
-#pragma unroll
-    for (int v = 0; v < VW; ++v) {
-      const int64_t j = rel + lane + 32 * v;
-      if (j >= 0 && j < Pp) prow[j] = acc[v];
+    if (lane == 0) {
+      // copies still in flight complete before the block's shared memory is released
+      for (int64_t r = q > kF1Stages ? q - kF1Stages : 0; r < q; ++r)
+        mbar_wait(&sh.full[(int)(r % kF1Stages)], (uint32_t)((r / kF1Stages) & 1), kMbarPolls);
+    }
+    return;
+  }
+
+  // ------------------------------------------------------------------ consumers
+  for (int u = blockIdx.x; u < a.nitems; u += gridDim.x) {
+    const Stage1Item it = a.items[u];
+    bool ok = false;
+    switch (it.pad2) {
+      case 8: ok = f1_consume<8>(a, sh, smf, it, warp, lane, st, par); break;
+      case 4: ok = f1_consume<4>(a, sh, smf, it, warp, lane, st, par); break;
+      default: ok = f1_consume<2>(a, sh, smf, it, warp, lane, st, par); break;
+    }
+    if (!ok) {
+      give_up();
+      return;
     }
   }
 }
@@ -398,6 +532,7 @@ int normalise_into(const tx_plan* p, const uint8_t* src, int64_t n, int64_t pitc
 }  // namespace
 
 int float_upload(tx_plan* p) {
+  TX_CUDA(raise_smem_limit((const void*)k_stage1_f32, kF1Smem));
   TX_CUDA(upload_stage2_pipe32<float>(p));
   return TX_OK;
 }
@@ -445,24 +580,26 @@ int float_execute(const tx_plan* p, tx_beam* b, const uint8_t* d_block, void* d_
   b->head = mod(b->head + p->T, p->R);
   if ((rc = mark(1))) return rc;
 
-  // stage 1: the plan's items (sub-band, coarse DMs, time tile), one block each
-  const int sw = p->tile_f + p->span_f + 4;
-  const int smem1 = p->m * sw * (int)sizeof(float);
-  const int nit = (int)p->items_f.size();
-#define TX_F1(VW)                                                                                                  \
-  do {                                                                                                             \
-    TX_CUDA(cudaFuncSetAttribute((const void*)k_stage1_f32<VW>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem1)); \
-    k_stage1_f32<VW><<<nit, kThreads1, smem1, st>>>(ring, p->R, start, p->dev.items_f, p->dev.d1, p->dev.abase,     \
-                                                   p->nchan, p->m, p->nsub, p->Pp, sw, P);                          \
-  } while (0)
-  switch (p->tile_f) {
-    case 256: TX_F1(8); break;
-    case 128: TX_F1(4); break;
-    case 64: TX_F1(2); break;
-    default: TX_F1(1); break;
-  }
-#undef TX_F1
-  TX_CUDA(cudaGetLastError());
+  // stage 1: the plan's items (sub-band, coarse DMs, time tile)
+  F1Args f1{};
+  f1.ring = ring;
+  f1.items = p->dev.items_f;
+  f1.chunks = p->dev.chunks_f;
+  f1.tab = p->dev.tab_f;
+  f1.abase = p->dev.abase;
+  f1.P = P;
+  f1.run = b->run;
+  f1.R = p->R;
+  f1.start = start;
+  f1.Pp = p->Pp;
+  f1.m = p->m;
+  f1.nsub = p->nsub;
+  f1.ndm = p->ndm;
+  f1.nitems = (int32_t)p->items_f.size();
+  f1.phase = p->phases_f == 1 ? 0 : (int32_t)(start & 3);
+  f1.polls = first_wait_polls();
+  TX_CUDA(launch_pdl(k_stage1_f32, dim3(std::min(f1.nitems, std::max(p->dev.num_sms, 1))), dim3(kF1Threads),
+                     (size_t)kF1Smem, st, f1));
   if ((rc = mark(2))) return rc;
 
   // stage 2 with per-tile sums

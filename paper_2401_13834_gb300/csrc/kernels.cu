@@ -82,6 +82,8 @@ int do_upload(tx_plan* p) {
   if ((rc = upload(&p->dev.tab1, p->tab1))) return rc;
   if ((rc = upload(&p->dev.tab2, p->tab2))) return rc;
   if ((rc = upload(&p->dev.items_f, p->items_f))) return rc;
+  if ((rc = upload(&p->dev.chunks_f, p->chunks_f))) return rc;
+  if ((rc = upload(&p->dev.tab_f, p->tab_f))) return rc;
   const int s1 = (int)stage1_smem_bytes(p->m, p->q1);
   switch (p->q1) {
     case 256: rc = set_stage1_attr_for<256>(p, s1); break;
@@ -230,6 +232,8 @@ void tx_plan_destroy(tx_plan* p) {
     cudaFree(p->dev.tab1);
     cudaFree(p->dev.tab2);
     cudaFree(p->dev.items_f);
+    cudaFree(p->dev.chunks_f);
+    cudaFree(p->dev.tab_f);
     cudaSetDevice(prev);
   }
   delete p;

@@ -79,6 +79,44 @@ static int auto_group(const std::vector<double>& f, double tsamp, int nsub, int 
   return g;
 }
 
+// Float path stage 1: outputs per lane of a warp for n coarse DMs. A warp sums
+// four consecutive coarse DMs over the tile (16 outputs per lane), or a half,
+// quarter or eighth of it where fewer coarse DMs would leave warps idle.
+static int32_t float_outputs(int n) {
+  const int quads = (n + kF1Quad - 1) / kF1Quad;
+  int vw = kF1Outputs;
+  while (vw > 2 && quads * (kF1Tile / 32 / vw) * 2 <= kF1Consumers) vw /= 2;
+  return vw;
+}
+
+// The chunks and offset tables of float stage 1 for sub-band s, coarse DMs
+// [kb, ke) (see tx_plan::chunks_f and tab_f); returns the number of chunks.
+static int32_t float_chunks(tx_plan* p, int s, int kb, int ke) {
+  const int m = p->m, nchan = p->nchan, n = ke - kb, quads = (n + kF1Quad - 1) / kF1Quad;
+  const int32_t* d1 = p->d1.data() + (size_t)s * m;      // d1[k * nchan + c]
+  int32_t nchunk = 0;
+  for (int c0 = 0; c0 < m; c0 += kF1Chan, ++nchunk) {
+    const int nc = std::min(kF1Chan, m - c0);
+    const int32_t words = quads * kF1Chan * kF1Quad / 2;
+    p->chunks_f.insert(p->chunks_f.end(), {(s * m + c0) * 32 + nc, words, (int32_t)(p->tab_f.size() / 4), 0, 0, 0, 0, 0});
+    for (int i = 0; i < kF1Rec - 8; ++i) p->chunks_f.push_back(i < nc ? d1[(size_t)kb * nchan + c0 + i] : 0);
+    for (int ph = 0; ph < p->phases_f; ++ph) {
+      const int phase = p->phases_f == 1 ? p->phase0_f : ph;
+      const size_t at = p->tab_f.size();
+      p->tab_f.resize(at + words, 0u);
+      for (int kk = 0; kk < quads * kF1Quad; ++kk)
+        for (int i = 0; i < nc; ++i) {
+          // past the last coarse DM: its offsets again (nothing is loaded or stored for them)
+          const int32_t d0 = d1[(size_t)kb * nchan + c0 + i];
+          const int32_t d = d1[(size_t)(kb + std::min(kk, n - 1)) * nchan + c0 + i] - d0;
+          const uint32_t v = (uint32_t)(i * kF1RawWords + ((phase + d0) & 3) + d);
+          p->tab_f[at + ((size_t)(kk / kF1Quad) * kF1Chan + i) * (kF1Quad / 2) + (kk % kF1Quad) / 2] |= v << (16 * (kk & 1));
+        }
+    }
+  }
+  return nchunk;
+}
+
 static int build(tx_plan* p, const tx_plan_desc* d) {
   // ---- validation ----------------------------------------------------------
   if (!d->freq_mhz || !d->dm || !d->widths) { set_error("null table pointer in plan description"); return TX_ERR_INVALID_ARG; }
@@ -363,14 +401,9 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
     return a.tau0 != b.tau0 ? a.tau0 < b.tau0 : (a.s != b.s ? a.s < b.s : a.kb < b.kb);
   });
   if (p->interm == TX_INTERM_F32) {
-    // float path stage 1: items of `tile_f` times whose coarse DMs' delay spread in
-    // the sub-band is at most span_f, the largest of four shapes whose staged
-    // float windows (tile + spread + 4 per channel) fit shared memory
-    const int shapes[4][2] = {{256, 240}, {128, 112}, {64, 48}, {32, 16}};
-    int si = 0;
-    while (si < 3 && (int64_t)m * (shapes[si][0] + shapes[si][1] + 4) * 4 > kSmemMax - 2048) ++si;
-    p->tile_f = shapes[si][0];
-    p->span_f = shapes[si][1];
+    // window starts are (head - L) mod R, head a multiple of 64 plus a multiple of T
+    p->phases_f = p->T % 4 == 0 ? 1 : 4;
+    p->phase0_f = (int32_t)((4 - p->L % 4) % 4);
     for (int s = 0; s < nsub; ++s) {
       int kb = 0;
       while (kb < nk) {
@@ -381,15 +414,19 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
           return v;
         };
         int ke = kb + 1;
-        while (ke < nk && ke - kb < kStage1MaxCoarse && spread(kb, ke + 1) <= p->span_f) ++ke;
+        while (ke < nk && ke - kb < kF1MaxCoarse && spread(kb, ke + 1) <= kF1Span) ++ke;
+        if (ke < nk && ke - kb > kF1Quad) ke = kb + (ke - kb) / kF1Quad * kF1Quad;   // whole warps
         int64_t lo = INT64_MAX, hi = 0;
         for (int k = kb; k < ke; ++k) {
           lo = std::min<int64_t>(lo, p->abase[(size_t)k * nsub + s]);
           hi = std::max<int64_t>(hi, (int64_t)p->abase[(size_t)k * nsub + s] + p->Pp);
         }
         const int32_t span = spread(kb, ke);
-        for (int64_t t0 = floor_div(lo, p->tile_f) * p->tile_f; t0 < hi; t0 += p->tile_f)
-          p->items_f.push_back(Stage1Item{s, kb, ke, (int32_t)t0, span, 0, 0, 0});
+        const size_t first = p->chunks_f.size() / kF1Rec;
+        if (p->tab_f.size() / 4 > (size_t)INT32_MAX) { set_error("float stage-1 tables too large"); return TX_ERR_UNSUPPORTED; }
+        const int32_t nchunk = float_chunks(p, s, kb, ke);
+        for (int64_t t0 = floor_div(lo, kF1Tile) * kF1Tile; t0 < hi; t0 += kF1Tile)
+          p->items_f.push_back(Stage1Item{s, kb, ke, (int32_t)t0, span, (int32_t)first, nchunk, float_outputs(ke - kb)});
         kb = ke;
       }
     }

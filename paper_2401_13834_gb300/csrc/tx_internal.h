@@ -54,6 +54,28 @@ constexpr int64_t stage2_pipe32_smem(int nst, int sc, int sw, int group) {
   return (int64_t)nst * ((int64_t)sc * sw + (int64_t)(group + 1) * ((sc + 3) & ~3)) * 4;
 }
 
+// ---- float path stage 1 -----------------------------------------------------
+// An item: one sub-band, up to kF1MaxCoarse coarse DMs whose delay spread in it
+// is at most kF1Span samples, kF1Tile times. Its channels are walked in chunks
+// of up to kF1Chan; a chunk's staged windows (kF1RawWords per channel) and its
+// offset table (kF1TabWords: 16 bits per coarse DM and channel) fill one of
+// kF1Stages stages.
+constexpr int kF1Tile = 512;
+constexpr int kF1Span = 240;
+constexpr int kF1Chan = 16;
+constexpr int kF1Quad = 4;             // consecutive coarse DMs summed by one warp
+constexpr int kF1Consumers = 20;       // consumer warps
+constexpr int kF1Outputs = 8;          // most outputs per lane and coarse DM
+constexpr int kF1MaxCoarse = kF1Consumers / (kF1Tile / 32 / kF1Outputs) * kF1Quad;
+constexpr int kF1Rec = 32;             // words of a chunk's record
+constexpr int kF1RawWords = kF1Tile + kF1Span + 8;
+constexpr int kF1TabWords = kF1MaxCoarse * kF1Chan / 2;
+constexpr int kF1Stages = 4;
+constexpr int kF1StageWords = kF1Chan * kF1RawWords + kF1TabWords;
+constexpr int kF1Smem = kF1Stages * kF1StageWords * 4;
+static_assert(kF1Smem <= kSmemMax - 1024, "float stage 1 shared memory");
+static_assert(kF1Chan * kF1RawWords < 65536, "float stage 1 offsets are 16 bits");
+
 // ---- matched filter ---------------------------------------------------------
 constexpr int kBoxTile = 2048;         // outputs per boxcar sub-tile (a unit holds 1, 2 or 4)
 constexpr int64_t kBoxMinUnits = 152 * 4 * 8;   // units a plan keeps for a full GPU before lengthening them
@@ -94,6 +116,8 @@ struct DevicePlan {
   int32_t* tab1 = nullptr;       // stage-1 offset tables of the item groups
   int32_t* tab2 = nullptr;       // pipelined stage 2: offset tables per (coarse group, sub-band chunk)
   Stage1Item* items_f = nullptr; // float path stage-1 items
+  int32_t* chunks_f = nullptr;   // their chunks
+  uint32_t* tab_f = nullptr;     // and the chunks' offset tables
 };
 
 void set_error(const char* fmt, ...);
@@ -149,8 +173,19 @@ struct tx_plan {
   int32_t e2w2 = 0;               // words of one stage-2 group's delays in shared memory (rounded to 4)
   int32_t box_tile = tx::kBoxTile;  // boxcar outputs per unit (a multiple of kBoxTile)
   int32_t ntile3 = 0;             // boxcar units per DM over [0, T)
-  int32_t tile_f = 0, span_f = 0;  // float path: stage-1 item length and delay spread limit
-  std::vector<tx::Stage1Item> items_f;  // float path stage-1 items (s, coarse DMs [kb, ke), times)
+  // float path stage-1 items: (s, coarse DMs [kb, ke), times); tab = first of
+  // its pad1 chunk records in chunks_f, pad2 = outputs per lane of a warp
+  std::vector<tx::Stage1Item> items_f;
+  // per (s, kb, ke) and chunk of channels, kF1Rec words: first channel * 32 +
+  // channels, words of its offset table, the table's place in tab_f (in 4
+  // words), then at word 8 the channels' delays d1[kb][c]
+  std::vector<int32_t> chunks_f;
+  // offset tables: per four coarse DMs kF1Chan x 4 16-bit words, the place of
+  // their first sample in the staged windows (channel * kF1RawWords +
+  // misalignment + d1[k][c] - d1[kb][c]); one table per residue mod 4 of an
+  // execute's window start (phases_f of them; 1 when every block has phase0_f)
+  std::vector<uint32_t> tab_f;
+  int32_t phases_f = 1, phase0_f = 0;
   std::vector<tx::Stage1Item> items1;
   // stage-1 offset tables, per (s, kb, ke): rows kk < ke - kb of (m + 3) & ~3
   // words, word c = c * staged words + ((tab1_phase + d1[kb][c]) & 15) +
