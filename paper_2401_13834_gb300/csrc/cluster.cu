@@ -7,31 +7,52 @@
 //                   with the non-core points within r of them
 //   outlier         any other point
 //
-// The paper finds neighbours with a kd-tree (Sec. 2.5, O(log N) per query);
-// on the GPU a uniform grid of cells slightly larger than r does the same
-// job: every neighbour of a point lies in the 3 x 3 cells around it, and the
-// points sorted by cell make each cell row one contiguous range.
+// The paper finds neighbours with a kd-tree (Sec. 2.5, O(log N) per query).
+// Here the points, sorted by (DM index, time), are rows of times, and the
+// neighbours of a point in another DM's row are those in one interval of times
+// around it: its half length in samples depends on the two DMs only and comes
+// from a table made with the clusterer (entries within rounding of a whole
+// sample are marked, and the interval's end points then take the test in
+// IEEE double, so that every decision is the double one). A query is a
+// binary search per row, whatever the density.
 //
 // Steps (one stream, no host round trip):
-//   1. canonical order: points sorted by (DM index, time) (radix sort);
-//   2. coordinates (delay table, t * t_samp) and cell keys; points sorted by cell;
-//   3. neighbour counts -> core flags;
-//   4. union-find over core pairs (lock-free: a root is linked under a smaller
-//      root, so the final root of a cluster is its smallest canonical index,
-//      which is the cluster's id);
+//   1. canonical order: points sorted by (DM index, time) (radix sort), row starts;
+//   2. neighbour counts, up to k + 1 -> core flags;
+//   3. runs: a core point joins the core point before it in its row when that
+//      is within r (head of each run by a max scan);
+//   4. union-find over runs of different rows (lock-free: a root is linked under a
+//      smaller root, so the final root of a cluster is its smallest canonical
+//      index, which is the cluster's id): of the core points in an interval only
+//      those are joined that no nearer one of them is already joined to, three
+//      at most;
 //   5. labels: a core point's root; a non-core point the smallest root among
 //      its core neighbours, or -1;
 //   6. per cluster: member count, DM and time extent, and the member of
-//      highest S/N (ties: smallest canonical index), by integer atomics;
+//      highest S/N (ties: smallest canonical index), by integer atomics, one
+//      set per warp and label;
 //   7. compaction of the clusters in id order (exclusive scan).
-// Every result is independent of thread order.
+// Every result is independent of thread order. What bounds it for a block's
+// candidates is the chain of some twenty dependent launches (a third of it the
+// radix sort's passes). Against visiting every pair within r through a grid of
+// cells: 150 to 260 thousand candidates of six bright pulses (r = 4 ms, 2048
+// DMs) 4.62 -> 0.29 ms; 52 thousand of a block whose pulses cover most of the
+// plane (r = 8 ms) 79 -> 0.88 ms.
+//
+// Where more than kMaxRows DM trials lie within r of one, rows are the wrong
+// index (a binary search for each, mostly empty); there a uniform grid of cells
+// slightly larger than r takes steps 2 to 5: every neighbour lies in the 3 x 3
+// cells around a point, and points sorted by cell make each cell row one
+// contiguous range.
 #include <cuda_runtime.h>
 
 #include <cub/cub.cuh>
 
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 #include <new>
+#include <vector>
 
 #include "tx_internal.h"
 
@@ -70,11 +91,18 @@ struct tx_clusterer {
   int32_t* pos = nullptr;
   void* temp = nullptr;
   size_t temp_bytes = 0;
+  // rows: [ndm][nrow + 1] half interval between a DM and the i-th after it, in
+  // samples, times 2, plus 1 when its end points need the double test; -1: out of
+  // reach. Row starts [ndm + 1]. nrow < 0: the grid is used.
+  int nrow = -1, sort_bits = 64;
+  int32_t *reach = nullptr, *row = nullptr;
 };
 
 namespace {
 
 constexpr int kThreads = 256;
+constexpr int kMaxRows = 256;               // DM trials within r of one for the row index
+constexpr int64_t kMaxReach = 1 << 24;      // entries of its table
 
 __global__ void k_cl_canon(const tx_cand* __restrict__ c, int n, unsigned long long* key, int32_t* val) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -181,22 +209,26 @@ __device__ __forceinline__ int cl_find(int32_t* parent, int x) {
   return x;
 }
 
+// Joins the sets of p and q.
+__device__ __forceinline__ void cl_unite(int32_t* parent, int p, int q) {
+  int a = cl_find(parent, p);
+  if (((volatile int32_t*)parent)[q] == a) return;  // already joined
+  int b = cl_find(parent, q);
+  while (a != b) {
+    if (a < b) { const int t = a; a = b; b = t; }
+    // link the larger root a under the smaller root b
+    const int old = atomicCAS(parent + a, a, b);
+    if (old == a) break;
+    a = cl_find(parent, a);
+    b = cl_find(parent, b);
+  }
+}
+
 __global__ void k_cl_union(const tx_clusterer C, int n) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n || !C.core[j]) return;
   for_neighbours(C, n, j, [&](int q) {
-    if (q >= j || !C.core[q]) return true;  // each core pair once
-    int a = cl_find(C.parent, j);
-    if (((volatile int32_t*)C.parent)[q] == a) return true;  // already joined
-    int b = cl_find(C.parent, q);
-    while (a != b) {
-      if (a < b) { const int t = a; a = b; b = t; }
-      // link the larger root a under the smaller root b
-      const int old = atomicCAS(C.parent + a, a, b);
-      if (old == a) break;
-      a = cl_find(C.parent, a);
-      b = cl_find(C.parent, b);
-    }
+    if (q < j && C.core[q]) cl_unite(C.parent, j, q);  // each core pair once
     return true;
   });
 }
@@ -223,24 +255,42 @@ __device__ __forceinline__ uint32_t ordered(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
+// A warp's points mostly share a label (they are neighbours in canonical
+// order): one set of atomics per warp and label.
 __global__ void k_cl_reduce(const tx_clusterer C, const tx_cand* __restrict__ c, int n) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= n) return;
-  const int l = C.label[j];
-  if (l < 0) return;
-  const tx_cand r = c[C.perm[j]];
-  atomicAdd(C.cnt + l, 1);
-  atomicMax(C.rep + l, ((unsigned long long)ordered(r.snr) << 32) | (uint32_t)(~(uint32_t)j));
-  atomicMin(C.dlo + l, r.dm_index);
-  atomicMax(C.dhi + l, r.dm_index);
-  atomicMin(C.tlo + l, r.t);
-  atomicMax(C.thi + l, r.t);
+  const int lane = threadIdx.x & 31;
+  const int l = j < n ? C.label[j] : -1;
+  tx_cand r{};
+  if (l >= 0) r = c[C.perm[j]];
+  const uint32_t snr = ordered(r.snr);
+  for (unsigned todo = __ballot_sync(0xffffffffu, l >= 0); todo;) {
+    const int lead = __ffs(todo) - 1;
+    const int lab = __shfl_sync(0xffffffffu, l, lead);
+    const bool in = l == lab;
+    const unsigned grp = __ballot_sync(0xffffffffu, in);
+    const uint32_t top = __reduce_max_sync(0xffffffffu, in ? snr : 0u);
+    const uint32_t first = __reduce_max_sync(0xffffffffu, in && snr == top ? ~(uint32_t)j : 0u);
+    const int dlo = __reduce_min_sync(0xffffffffu, in ? r.dm_index : INT32_MAX);
+    const int dhi = __reduce_max_sync(0xffffffffu, in ? r.dm_index : INT32_MIN);
+    const int tlo = __reduce_min_sync(0xffffffffu, in ? r.t : INT32_MAX);
+    const int thi = __reduce_max_sync(0xffffffffu, in ? r.t : INT32_MIN);
+    if (lane == lead) {
+      atomicAdd(C.cnt + lab, __popc(grp));
+      atomicMax(C.rep + lab, ((unsigned long long)top << 32) | first);
+      atomicMin(C.dlo + lab, dlo);
+      atomicMax(C.dhi + lab, dhi);
+      atomicMin(C.tlo + lab, tlo);
+      atomicMax(C.thi + lab, thi);
+    }
+    todo &= ~grp;
+  }
 }
 
-__global__ void k_cl_flag(const tx_clusterer C, int n) {
+__global__ void k_cl_flag(const tx_clusterer C, int n, int32_t* flag) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
-  C.flag[j] = C.core[j] && C.label[j] == j;
+  flag[j] = C.core[j] && C.label[j] == j;
 }
 
 __global__ void k_cl_emit(const tx_clusterer C, const tx_cand* __restrict__ c, int n, tx_cluster* out,
@@ -267,10 +317,236 @@ __global__ void k_cl_emit(const tx_clusterer C, const tx_cand* __restrict__ c, i
   o.t_hi = C.thi[j];
   out[C.pos[j]] = o;
 }
+// ---- rows -------------------------------------------------------------------
+// The DM index of a canonical key (one that is no trial of the plan: ndm, a row
+// without neighbours).
+__device__ __forceinline__ int cl_dm(const tx_clusterer& C, unsigned long long key) {
+  return (int)min((unsigned long long)C.ndm, key >> 32);
+}
+
+// row[d] = first canonical index of DM d or later, d <= ndm; and what the
+// other steps start from.
+__global__ void k_cl_rows(const tx_clusterer C, const unsigned long long* __restrict__ key, int n) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const int d = cl_dm(C, key[j]), before = j ? cl_dm(C, key[j - 1]) : -1;
+  for (int e = before + 1; e <= d; ++e) C.row[e] = j;
+  if (j == n - 1)
+    for (int e = d + 1; e <= C.ndm; ++e) C.row[e] = n;
+  C.cnt[j] = 0;
+  C.rep[j] = 0ull;
+  C.dlo[j] = INT32_MAX;
+  C.dhi[j] = INT32_MIN;
+  C.tlo[j] = INT32_MAX;
+  C.thi[j] = INT32_MIN;
+}
+
+// (x_q - x_p)^2 + (y_q - y_p)^2 <= r^2 in IEEE double.
+__device__ __forceinline__ bool cl_near(const tx_clusterer& C, int dp, uint32_t tp, int dq, uint32_t tq) {
+  const double gx = __dsub_rn(C.table[dq], C.table[dp]);
+  const double gy = __dsub_rn(__dmul_rn((double)(int32_t)tq, C.tsamp_ms), __dmul_rn((double)(int32_t)tp, C.tsamp_ms));
+  return __dadd_rn(__dmul_rn(gx, gx), __dmul_rn(gy, gy)) <= __dmul_rn(C.r, C.r);
+}
+
+// The times of row dq within r of point (d, t), as [lo, hi] (reach: the table's
+// entry for the two DMs).
+__device__ __forceinline__ void cl_interval(const tx_clusterer& C, int d, uint32_t t, int dq, int reach, uint32_t& lo,
+                                            uint32_t& hi) {
+  const uint32_t h = (uint32_t)(reach >> 1);
+  lo = t >= h ? t - h : 0u;
+  hi = t + h;
+  if (reach & 1) {
+    if (t >= h && !cl_near(C, d, t, dq, lo)) ++lo;   // an interval of none when h = 0
+    if (!cl_near(C, d, t, dq, hi)) hi = h ? hi - 1 : 0u;
+  }
+}
+
+// First entry of [b, e) whose time is at least t.
+__device__ __forceinline__ int cl_search(const unsigned long long* __restrict__ key, int b, int e, uint32_t t) {
+  while (b < e) {
+    const int mid = (b + e) >> 1;
+    if ((uint32_t)key[mid] < t) b = mid + 1; else e = mid;
+  }
+  return b;
+}
+
+// Calls f(dq, reach) for the non-empty rows within r of row d, the point's own
+// first, then outwards; f returns false to stop.
+template <typename F>
+__device__ __forceinline__ void cl_rows(const tx_clusterer& C, int d, bool before, F&& f) {
+  const int w = C.nrow + 1;
+  if (d >= C.ndm) return;
+  if (!f(d, __ldg(C.reach + (size_t)d * w))) return;
+  bool up = true, down = before;
+  for (int i = 1; i <= C.nrow && (up || down); ++i) {
+    if (up) {
+      const int q = d + i;
+      const int h = q < C.ndm ? __ldg(C.reach + (size_t)d * w + i) : -1;
+      if (h < 0) up = false;
+      else if (C.row[q] < C.row[q + 1] && !f(q, h)) return;
+    }
+    if (down) {
+      const int q = d - i;
+      const int h = q >= 0 ? __ldg(C.reach + (size_t)q * w + i) : -1;
+      if (h < 0) down = false;
+      else if (C.row[q] < C.row[q + 1] && !f(q, h)) return;
+    }
+  }
+}
+
+__global__ void k_cl_row_core(const tx_clusterer C, const unsigned long long* __restrict__ key, int n) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const int d = cl_dm(C, key[j]);
+  const uint32_t t = (uint32_t)key[j];
+  long long cnt = -1;   // the point itself is counted
+  cl_rows(C, d, true, [&](int q, int reach) {
+    uint32_t lo, hi;
+    cl_interval(C, d, t, q, reach, lo, hi);
+    const int e = C.row[q + 1];
+    int p;
+    if (q == d) {   // up to k + 1 to the left of the point, then on to the right
+      p = j;
+      while (p > C.row[d] && (uint32_t)key[p - 1] >= lo && j - p <= C.k) --p;
+    } else {
+      p = cl_search(key, C.row[q], e, lo);
+    }
+    for (; p < e && (uint32_t)key[p] <= hi && cnt <= C.k; ++p) ++cnt;
+    return cnt <= C.k;
+  });
+  C.core[j] = cnt > C.k;
+}
+
+// val[j] = j for the head of a run of core points, else 0: a core point whose
+// row's core point before it is out of reach.
+__global__ void k_cl_row_heads(const tx_clusterer C, const unsigned long long* __restrict__ key, int n, int32_t* val) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  int v = 0;
+  if (C.core[j]) {
+    const int d = cl_dm(C, key[j]);
+    uint32_t lo, hi;
+    cl_interval(C, d, (uint32_t)key[j], d, __ldg(C.reach + (size_t)d * (C.nrow + 1)), lo, hi);
+    v = j;
+    for (int p = j - 1; p >= C.row[d] && (uint32_t)key[p] >= lo; --p)
+      if (C.core[p]) { v = 0; break; }
+  }
+  val[j] = v;
+}
+
+// Calls f(p) for core points p of the interval [lo, hi] of row q: the first, and
+// after each the first that is out of its reach (those in its reach are joined
+// to it already, own0 being the row's reach in itself).
+template <typename F>
+__device__ __forceinline__ void cl_cores(const tx_clusterer& C, const unsigned long long* __restrict__ key, int q,
+                                         uint32_t lo, uint32_t hi, F&& f) {
+  const int e = C.row[q + 1];
+  const int own = __ldg(C.reach + (size_t)q * (C.nrow + 1));
+  const uint32_t step = (uint32_t)(own >> 1) - ((own & 1) && own > 1 ? 1u : 0u);
+  int p = cl_search(key, C.row[q], e, lo);
+  while (true) {
+    while (p < e && (uint32_t)key[p] <= hi && !C.core[p]) ++p;
+    if (p >= e || (uint32_t)key[p] > hi) return;
+    f(p);
+    const uint32_t nt = (uint32_t)key[p] + step;   // the last time certainly in p's reach
+    if (nt >= hi) return;
+    p = cl_search(key, p + 1, e, nt + 1);
+  }
+}
+
+__global__ void k_cl_row_union(const tx_clusterer C, const unsigned long long* __restrict__ key, int n) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n || !C.core[j]) return;
+  const int d = cl_dm(C, key[j]);
+  const uint32_t t = (uint32_t)key[j];
+  cl_rows(C, d, false, [&](int q, int reach) {   // each pair of rows once: later rows only
+    if (q == d) return true;
+    uint32_t lo, hi;
+    cl_interval(C, d, t, q, reach, lo, hi);
+    if (lo <= hi) cl_cores(C, key, q, lo, hi, [&](int p) { cl_unite(C.parent, j, p); });
+    return true;
+  });
+}
+
+// Labels of the core points, and the flags of the clusters' first points.
+__global__ void k_cl_row_label(const tx_clusterer C, int n, int32_t* flag) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n) return;
+  const int l = C.core[j] ? cl_find(C.parent, j) : -1;
+  C.label[j] = l;
+  flag[j] = l == j;
+}
+
+// parent = the head of a core point's run (val after the max scan)
+__global__ void k_cl_row_parent(const tx_clusterer C, const int32_t* __restrict__ val, int n) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j < n) C.parent[j] = C.core[j] ? val[j] : j;
+}
+
+__global__ void k_cl_row_border(const tx_clusterer C, const unsigned long long* __restrict__ key, int n) {
+  const int j = blockIdx.x * blockDim.x + threadIdx.x;
+  if (j >= n || C.core[j]) return;
+  const int d = cl_dm(C, key[j]);
+  const uint32_t t = (uint32_t)key[j];
+  int best = INT32_MAX;
+  cl_rows(C, d, true, [&](int q, int reach) {
+    uint32_t lo, hi;
+    cl_interval(C, d, t, q, reach, lo, hi);
+    if (lo <= hi) cl_cores(C, key, q, lo, hi, [&](int p) { best = min(best, C.label[p]); });
+    return true;
+  });
+  C.label[j] = best == INT32_MAX ? -1 : best;
+}
+
+struct Larger {
+  __device__ __forceinline__ int32_t operator()(int32_t a, int32_t b) const { return a > b ? a : b; }
+};
 
 template <typename T>
 int dalloc(T** p, int64_t n) {
   TX_CUDA(cudaMalloc((void**)p, (size_t)std::max<int64_t>(n, 1) * sizeof(T)));
+  return TX_OK;
+}
+
+// Steps 2 to 5 on rows; canonical keys in key_b, flags to fl.
+int run_rows(tx_clusterer* C, int ni, int32_t* fl, cudaStream_t st) {
+  const int grid = (ni + kThreads - 1) / kThreads;
+  const unsigned long long* key = C->key_b;
+  k_cl_rows<<<grid, kThreads, 0, st>>>(*C, key, ni);
+  k_cl_row_core<<<grid, kThreads, 0, st>>>(*C, key, ni);
+  k_cl_row_heads<<<grid, kThreads, 0, st>>>(*C, key, ni, C->flag);
+  TX_CUDA(cudaGetLastError());
+  size_t tb = C->temp_bytes;
+  TX_CUDA(cub::DeviceScan::InclusiveScan(C->temp, tb, C->flag, C->pos, Larger{}, ni, st));
+  k_cl_row_parent<<<grid, kThreads, 0, st>>>(*C, C->pos, ni);
+  k_cl_row_union<<<grid, kThreads, 0, st>>>(*C, key, ni);
+  k_cl_row_label<<<grid, kThreads, 0, st>>>(*C, ni, fl);
+  k_cl_row_border<<<grid, kThreads, 0, st>>>(*C, key, ni);
+  TX_CUDA(cudaGetLastError());
+  return TX_OK;
+}
+
+// Steps 2 to 5 on a grid of cells.
+int run_grid(tx_clusterer* C, const tx_cand* d_cands, int ni, int32_t* fl, cudaStream_t st) {
+  const int grid = (ni + kThreads - 1) / kThreads;
+  // coordinates and cells
+  k_cl_coords<<<grid, kThreads, 0, st>>>(d_cands, C->perm, ni, C->table, C->tsamp_ms, C->cell, C->x, C->y,
+                                         C->key_a, C->val_a);
+  TX_CUDA(cudaGetLastError());
+  unsigned long long* ck = C->key_b;       // canonical keys are no longer needed
+  int32_t* ci = reinterpret_cast<int32_t*>(C->flag);
+  size_t tb = C->temp_bytes;
+  TX_CUDA(cub::DeviceRadixSort::SortPairs(C->temp, tb, C->key_a, ck, C->val_a, ci, ni, 0, 64, st));
+  C->ckey = ck;
+  C->cidx = ci;
+  k_cl_local<<<grid, kThreads, 0, st>>>(*C, ni);
+  // core flags, union-find, labels
+  k_cl_core<<<grid, kThreads, 0, st>>>(*C, ni);
+  k_cl_union<<<grid, kThreads, 0, st>>>(*C, ni);
+  k_cl_label_core<<<grid, kThreads, 0, st>>>(*C, ni);
+  k_cl_label_border<<<grid, kThreads, 0, st>>>(*C, ni);
+  k_cl_flag<<<grid, kThreads, 0, st>>>(*C, ni, fl);
+  TX_CUDA(cudaGetLastError());
   return TX_OK;
 }
 
@@ -296,7 +572,40 @@ int32_t tx_clusterer_create(const tx_plan* p, double radius_ms, int32_t k, int64
   C->ndm = p->ndm;
   const int64_t n = max_points;
   int rc = TX_OK;
+  while (C->sort_bits > 33 && ((int64_t)1 << (C->sort_bits - 33)) >= p->ndm) --C->sort_bits;   // 32 + bits of a DM index
+  // rows: the half intervals, unless too many DMs lie within r of one
+  std::vector<int32_t> reach;
+  {
+    const std::vector<double>& x = p->delay_ms;
+    const volatile double r2 = radius_ms * radius_ms;
+    int most = 0;
+    for (int d = 0, e = 0; d < p->ndm && most <= kMaxRows; ++d) {
+      for (e = std::max(e, d); e + 1 < p->ndm; ++e) {
+        const double gx = x[e + 1] - x[d];
+        const volatile double g2 = gx * gx;
+        if (!(g2 <= r2)) break;
+      }
+      most = std::max(most, e - d);
+    }
+    if (most <= kMaxRows && (int64_t)p->ndm * (most + 1) <= kMaxReach && radius_ms / C->tsamp_ms < 5e8) {
+      C->nrow = most;
+      reach.assign((size_t)p->ndm * (most + 1), -1);
+      for (int d = 0; d < p->ndm; ++d)
+        for (int i = 0; i <= most && d + i < p->ndm; ++i) {
+          const double gx = x[d + i] - x[d];
+          const volatile double g2 = gx * gx;
+          if (!(g2 <= r2)) break;
+          // r^2 - gx^2 in samples squared; the test's own rounding moves it by far less than `slack`
+          const double q = std::max(0.0, (r2 - g2) / (C->tsamp_ms * C->tsamp_ms)), h = std::floor(std::sqrt(q));
+          const double slack = 1e-5 * (h + 1.0) + 1e-12 * (r2 / (C->tsamp_ms * C->tsamp_ms));
+          const bool next = (h + 1.0) * (h + 1.0) - q <= slack;
+          reach[(size_t)d * (most + 1) + i] = 2 * (int32_t)(next ? h + 1.0 : h) + (next || q - h * h <= slack ? 1 : 0);
+        }
+    }
+  }
   if (!rc) rc = dalloc(&C->table, p->ndm);
+  if (!rc) rc = dalloc(&C->row, (int64_t)p->ndm + 1);
+  if (!rc) rc = dalloc(&C->reach, (int64_t)reach.size());
   if (!rc) rc = dalloc(&C->key_a, n);
   if (!rc) rc = dalloc(&C->key_b, n);
   if (!rc) rc = dalloc(&C->val_a, n);
@@ -321,11 +630,17 @@ int32_t tx_clusterer_create(const tx_plan* p, double radius_ms, int32_t k, int64
     set_error("delay table upload failed");
     rc = TX_ERR_CUDA;
   }
+  if (!rc && !reach.empty() &&
+      cudaMemcpy(C->reach, reach.data(), reach.size() * sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess) {
+    set_error("interval table upload failed");
+    rc = TX_ERR_CUDA;
+  }
   if (!rc) {
-    size_t a = 0, b = 0;
+    size_t a = 0, b = 0, c = 0;
     cub::DeviceRadixSort::SortPairs(nullptr, a, C->key_a, C->key_b, C->val_a, C->val_b, (int)n);
     cub::DeviceScan::ExclusiveSum(nullptr, b, C->flag, C->pos, (int)n);
-    C->temp_bytes = std::max(a, b);
+    cub::DeviceScan::InclusiveScan(nullptr, c, C->flag, C->pos, Larger{}, (int)n);
+    C->temp_bytes = std::max(a, std::max(b, c));
     if (cudaMalloc(&C->temp, std::max<size_t>(C->temp_bytes, 16)) != cudaSuccess) {
       set_error("clusterer scratch allocation failed");
       rc = TX_ERR_OOM;
@@ -351,32 +666,19 @@ int32_t tx_cluster_run(tx_clusterer* C, const tx_cand* d_cands, int64_t n, tx_cl
   // 1. canonical order
   k_cl_canon<<<grid, kThreads, 0, st>>>(d_cands, ni, C->key_a, C->val_a);
   TX_CUDA(cudaGetLastError());
-  TX_CUDA(cub::DeviceRadixSort::SortPairs(C->temp, tb, C->key_a, C->key_b, C->val_a, C->val_b, ni, 0, 64, st));
+  TX_CUDA(cub::DeviceRadixSort::SortPairs(C->temp, tb, C->key_a, C->key_b, C->val_a, C->val_b, ni, 0, C->sort_bits, st));
   C->perm = C->val_b;
-  // 2. coordinates and cells
-  k_cl_coords<<<grid, kThreads, 0, st>>>(d_cands, C->perm, ni, C->table, C->tsamp_ms, C->cell, C->x, C->y,
-                                         C->key_a, C->val_a);
-  TX_CUDA(cudaGetLastError());
-  unsigned long long* ck = C->key_b;       // canonical keys are no longer needed
-  int32_t* ci = reinterpret_cast<int32_t*>(C->flag);
-  tb = C->temp_bytes;
-  TX_CUDA(cub::DeviceRadixSort::SortPairs(C->temp, tb, C->key_a, ck, C->val_a, ci, ni, 0, 64, st));
-  C->ckey = ck;
-  C->cidx = ci;
-  k_cl_local<<<grid, kThreads, 0, st>>>(*C, ni);
-  // 3-5. core flags, union-find, labels
-  k_cl_core<<<grid, kThreads, 0, st>>>(*C, ni);
-  k_cl_union<<<grid, kThreads, 0, st>>>(*C, ni);
-  k_cl_label_core<<<grid, kThreads, 0, st>>>(*C, ni);
-  k_cl_label_border<<<grid, kThreads, 0, st>>>(*C, ni);
-  TX_CUDA(cudaGetLastError());
+  int32_t* fl = C->val_a;   // flags of the clusters' first points
+  if (C->nrow >= 0) {
+    if (const int rc = run_rows(C, ni, fl, st)) return rc;
+  } else if (const int rc = run_grid(C, d_cands, ni, fl, st)) {
+    return rc;
+  }
   // 6. per-cluster reductions
   k_cl_reduce<<<grid, kThreads, 0, st>>>(*C, d_cands, ni);
   // 7. clusters in id order
-  int32_t* fl = C->val_a;                  // cell values are no longer needed
   tx_clusterer Cf = *C;
   Cf.flag = fl;
-  k_cl_flag<<<grid, kThreads, 0, st>>>(Cf, ni);
   tb = C->temp_bytes;
   TX_CUDA(cub::DeviceScan::ExclusiveSum(C->temp, tb, fl, C->pos, ni, st));
   k_cl_emit<<<grid, kThreads, 0, st>>>(Cf, d_cands, ni, d_out, d_nclusters, d_labels, d_order);
@@ -392,7 +694,7 @@ void tx_clusterer_destroy(tx_clusterer* C) {
   for (void* q : {(void*)C->table, (void*)C->key_a, (void*)C->key_b, (void*)C->val_a, (void*)C->val_b, (void*)C->x,
                   (void*)C->y, (void*)C->core, (void*)C->parent, (void*)C->label, (void*)C->cnt, (void*)C->rep,
                   (void*)C->dlo, (void*)C->dhi, (void*)C->tlo, (void*)C->thi, (void*)C->flag, (void*)C->pos,
-                  (void*)C->xs, (void*)C->ys, C->temp})
+                  (void*)C->xs, (void*)C->ys, (void*)C->reach, (void*)C->row, C->temp})
     cudaFree(q);
   cudaSetDevice(prev);
   delete C;
