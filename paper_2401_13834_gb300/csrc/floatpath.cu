@@ -305,9 +305,14 @@ __global__ void __launch_bounds__(kF1Threads, 1) k_stage1_f32(const F1Args a) {
         const int64_t pa = p & ~(int64_t)3;
         const float* row = a.ring + (size_t)(c0 + lane) * a.R;
         float* d = dst + lane * kF1RawWords;
-        const int first = (int)min((int64_t)words, a.R - pa);
-        bulk_g2s(d, row + pa, (uint32_t)first * 4u, &sh.full[st]);
-        if (first < words) bulk_g2s(d + first, row, (uint32_t)(words - first) * 4u, &sh.full[st]);
+        // in pieces where the window wraps the ring's end (a short ring more than once)
+        int64_t from = pa;
+        for (int done = 0; done < words;) {
+          const int len = (int)min((int64_t)(words - done), a.R - from);
+          bulk_g2s(d + done, row + from, (uint32_t)len * 4u, &sh.full[st]);
+          done += len;
+          from = 0;
+        }
       }
       if (lane == 31)
         bulk_g2s(dst + kF1Chan * kF1RawWords, a.tab + (size_t)to * 4 + (size_t)a.phase * tw, (uint32_t)tw * 4u,
