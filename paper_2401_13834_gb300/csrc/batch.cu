@@ -75,6 +75,7 @@ struct BatchLaunch {
   int kind = 0;
   int wave = 0;
   int q1 = 0, split = 0, nwc = 0, mode = 0, half = 0, pipe = 0;  // template selectors
+  Wide1Shape s1w{};                          // wide sub-bands' stage 1 (nst > 0)
   int grid = 0, threads = 0, smem = 0;
   int nmem = 0, nunits = 0;                  // member beams, work units (stage 1: the plans' items)
   int64_t off = 0, mem = 0;                  // offsets of the unit-offset / member arrays in the table
@@ -121,6 +122,11 @@ const void* launch_kernel(const BatchLaunch& L) {
     case kTailOut: return (const void*)k_tail<SlotArgs>;
     case kOffsets: return (const void*)k_offsets<SlotArgs>;
     case kStage1:
+      if (L.s1w.nst) {
+#define TX_KW(VW) (L.half ? (const void*)k_stage1_wide<VW, uint16_t, SlotArgs, true> : (const void*)k_stage1_wide<VW, uint16_t, SlotArgs>)
+        return L.s1w.vw == 8 ? TX_KW(8) : L.s1w.vw == 4 ? TX_KW(4) : TX_KW(2);
+#undef TX_KW
+      }
 #define TX_K1(Q) (L.half ? (const void*)k_stage1<Q, uint16_t, SlotArgs, true> : (const void*)k_stage1<Q, uint16_t, SlotArgs>)
       switch (L.q1) {
         case 256: return TX_K1(256);
@@ -249,9 +255,9 @@ int build_batch(tx_batch* B, int64_t budget) {
     // ---- stage 1, one launch per (tile length, channels per sub-band): the shared
     // memory of a launch is laid out for its largest sub-band, and a mix would
     // take carve-out from L1 for the smaller ones
-    std::map<std::tuple<int, int, int>, std::vector<int>> by_q;
+    std::map<std::tuple<int, int, int, int>, std::vector<int>> by_q;
     for (int b : mem)
-      by_q[{B->plans[b]->q1, B->plans[b]->m, B->plans[b]->interm == TX_INTERM_F16}].push_back(b);
+      by_q[{B->plans[b]->q1, B->plans[b]->m, B->plans[b]->interm == TX_INTERM_F16, B->plans[b]->wide1 ? B->plans[b]->s1w.vw : 0}].push_back(b);
     for (auto& kv : by_q) {
       BatchLaunch L;
       L.kind = kStage1;
@@ -262,9 +268,10 @@ int build_batch(tx_batch* B, int64_t budget) {
         return rc;
       L.layout = std::get<1>(kv.first);  // channels per sub-band of every member
       const int mL = L.layout;
-      L.smem = (int)stage1_smem_bytes(mL, L.q1);
+      if (std::get<3>(kv.first)) L.s1w = B->plans[kv.second[0]]->s1w;   // channels and words per lane give the shape
+      L.smem = L.s1w.nst ? L.s1w.smem() : (int)stage1_smem_bytes(mL, L.q1);
       if (L.smem > kSmemMax) { set_error("stage-1 shared memory for %d channels per sub-band exceeds the limit", mL); return TX_ERR_UNSUPPORTED; }
-      L.threads = kStage1Warps * 32;
+      L.threads = (L.s1w.nst ? kWide1Warps : kStage1Warps) * 32;
       L.grid = std::min(L.nunits, nsm);
       L.ctr = (int64_t)tab.size();
       tab.push_back(0);
@@ -427,6 +434,24 @@ int enqueue(tx_batch* B, const BeamArgs* h_src, cudaStream_t st) {
       case kStage1: {
         int32_t* ictr = B->d_tab + L.ctr;
         TX_CUDA(cudaMemsetAsync(ictr, 0, sizeof(int32_t), st));
+        if (L.s1w.nst) {
+#define TX_BW(VW)                                                                                               \
+  do {                                                                                                           \
+    if (L.half)                                                                                                  \
+      k_stage1_wide<VW, uint16_t, SlotArgs, true><<<L.grid, L.threads, L.smem, st>>>(src, off, mem, L.nmem,       \
+                                                                                     L.nunits, L.s1w, 1u, ictr); \
+    else                                                                                                         \
+      k_stage1_wide<VW, uint16_t, SlotArgs><<<L.grid, L.threads, L.smem, st>>>(src, off, mem, L.nmem, L.nunits,   \
+                                                                               L.s1w, 1u, ictr);                 \
+  } while (0)
+          switch (L.s1w.vw) {
+            case 8: TX_BW(8); break;
+            case 4: TX_BW(4); break;
+            default: TX_BW(2); break;
+          }
+#undef TX_BW
+          break;
+        }
 #define TX_B1(Q)                                                                                                \
   do {                                                                                                           \
     if (L.half)                                                                                                  \

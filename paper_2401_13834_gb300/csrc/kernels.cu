@@ -68,6 +68,14 @@ int set_stage1_attr_for(const tx_plan* p, int bytes) {
   return set_stage1_attr<Q, int32_t>(bytes);
 }
 
+// The wide sub-bands' stage 1 for words per lane vw (8, 4 or 2).
+template <int VW>
+const void* wide1_kernel_vw(int interm) {
+  if (interm == TX_INTERM_F16) return (const void*)k_stage1_wide<VW, uint16_t, OneBeam, true>;
+  return interm == TX_INTERM_U16 ? (const void*)k_stage1_wide<VW, uint16_t, OneBeam>
+                                 : (const void*)k_stage1_wide<VW, int32_t, OneBeam>;
+}
+
 int do_upload(tx_plan* p) {
   int dev = 0;
   TX_CUDA(cudaGetDevice(&dev));
@@ -84,6 +92,11 @@ int do_upload(tx_plan* p) {
   if ((rc = upload(&p->dev.items_f, p->items_f))) return rc;
   if ((rc = upload(&p->dev.chunks_f, p->chunks_f))) return rc;
   if ((rc = upload(&p->dev.tab_f, p->tab_f))) return rc;
+  if (p->wide1)
+    TX_CUDA(raise_smem_limit(p->s1w.vw == 8   ? wide1_kernel_vw<8>(p->interm)
+                             : p->s1w.vw == 4 ? wide1_kernel_vw<4>(p->interm)
+                                              : wide1_kernel_vw<2>(p->interm),
+                             p->s1w.smem()));
   const int s1 = (int)stage1_smem_bytes(p->m, p->q1);
   switch (p->q1) {
     case 256: rc = set_stage1_attr_for<256>(p, s1); break;
@@ -123,6 +136,28 @@ void launch_stage1_t(const tx_plan* p, const BeamArgs& a, int32_t* ictr, cudaStr
   const int grid = std::min(nitems, std::max(p->dev.num_sms, 1));
   launch_pdl(k_stage1<Q, PT, OneBeam, HALF>, grid, kStage1Warps * 32, (size_t)stage1_smem_bytes(p->m, Q), st,
              OneBeam{a}, nullptr, nullptr, 1, nitems, p->m, 1u, ictr);
+}
+
+template <int VW, typename PT, bool HALF = false>
+void launch_wide1_t(const tx_plan* p, const BeamArgs& a, int32_t* ictr, cudaStream_t st, bool pdl) {
+  const int nitems = (int)p->items1.size();
+  const int grid = std::min(nitems, std::max(p->dev.num_sms, 1));
+  if (pdl)
+    launch_pdl(k_stage1_wide<VW, PT, OneBeam, HALF>, grid, kWide1Warps * 32, (size_t)p->s1w.smem(), st, OneBeam{a},
+               nullptr, nullptr, 1, nitems, p->s1w, 1u, ictr);
+  else
+    k_stage1_wide<VW, PT, OneBeam, HALF><<<grid, kWide1Warps * 32, p->s1w.smem(), st>>>(
+        OneBeam{a}, nullptr, nullptr, 1, nitems, p->s1w, 1u, ictr);
+}
+
+// stage 1 of a plan of wide sub-bands with its item counter
+template <typename PT, bool HALF = false>
+void launch_wide1(const tx_plan* p, const BeamArgs& a, int32_t* ictr, cudaStream_t st, bool pdl = true) {
+  switch (p->s1w.vw) {
+    case 8: launch_wide1_t<8, PT, HALF>(p, a, ictr, st, pdl); break;
+    case 4: launch_wide1_t<4, PT, HALF>(p, a, ictr, st, pdl); break;
+    default: launch_wide1_t<2, PT, HALF>(p, a, ictr, st, pdl); break;
+  }
 }
 
 // stage 1 with its item counter `ictr` (zeroed before, by the ingest)
@@ -450,7 +485,11 @@ int execute_impl(const tx_plan* p, tx_beam* b, const uint8_t* d_block, void* d_o
   }
 
   // stage 1
-  switch (p->q1) {
+  if (p->wide1) {
+    if (half) launch_wide1<uint16_t, true>(p, a, ictr, st);
+    else if (p->interm == TX_INTERM_U16) launch_wide1<uint16_t>(p, a, ictr, st);
+    else launch_wide1<int32_t>(p, a, ictr, st);
+  } else switch (p->q1) {
     case 256: rc = launch_stage1<256>(p, a, ictr, st); break;
     case 128: rc = launch_stage1<128>(p, a, ictr, st); break;
     case 64: rc = launch_stage1<64>(p, a, ictr, st); break;
@@ -854,7 +893,9 @@ int32_t tx_dedisperse_noalloc(const tx_plan* p, const uint8_t* d_x, int64_t ld, 
     k_stage1<Q, uint16_t, OneBeam><<<grid1, kStage1Warps * 32, smem1, st>>>(OneBeam{a}, nullptr, nullptr, 1, nitems, \
                                                                             p->m, 1u, ictr);                  \
   } while (0)
-  switch (p->q1) {
+  if (p->wide1) {
+    launch_wide1<uint16_t>(p, a, ictr, st, false);
+  } else switch (p->q1) {
     case 256: TX_NA_S1(256); break;
     case 128: TX_NA_S1(128); break;
     case 64: TX_NA_S1(64); break;

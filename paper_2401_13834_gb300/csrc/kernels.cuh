@@ -794,6 +794,341 @@ k_stage1(const Src src, const int32_t* __restrict__ uoff, const int32_t* __restr
 }
 
 // ---------------------------------------------------------------------------
+// stage 1 of wide sub-bands
+// ---------------------------------------------------------------------------
+// Adds `cnt` channels' words to the sums: aw the words themselves, ah their odd
+// bytes as 16-bit lanes. e: the channels' byte offsets (16-byte aligned).
+template <int VW>
+__device__ __forceinline__ void wide1_add(uint32_t (&aw)[VW], uint32_t (&ah)[VW], const uint8_t* __restrict__ base,
+                                           const uint32_t* __restrict__ e, int cnt, uint32_t one) {
+  int c = 0;
+  for (; c + 3 < cnt; c += 4) {
+    const uint4 o = *reinterpret_cast<const uint4*>(e + c);
+    const uint32_t* r0 = reinterpret_cast<const uint32_t*>(base + o.x);
+    const uint32_t* r1 = reinterpret_cast<const uint32_t*>(base + o.y);
+    const uint32_t* r2 = reinterpret_cast<const uint32_t*>(base + o.z);
+    const uint32_t* r3 = reinterpret_cast<const uint32_t*>(base + o.w);
+#pragma unroll
+    for (int v = 0; v < VW; ++v) {
+      const uint32_t w0 = r0[32 * v], w1 = r1[32 * v], w2 = r2[32 * v], w3 = r3[32 * v];
+      madd(aw[v], w0, one);
+      madd(aw[v], w1, one);
+      madd(aw[v], w2, one);
+      madd(aw[v], w3, one);
+      ah[v] += __byte_perm(w0, 0u, 0x4341) + __byte_perm(w1, 0u, 0x4341);
+      ah[v] += __byte_perm(w2, 0u, 0x4341) + __byte_perm(w3, 0u, 0x4341);
+    }
+  }
+  if (cnt & 2) {
+    const uint2 o = *reinterpret_cast<const uint2*>(e + c);
+    const uint32_t* r0 = reinterpret_cast<const uint32_t*>(base + o.x);
+    const uint32_t* r1 = reinterpret_cast<const uint32_t*>(base + o.y);
+#pragma unroll
+    for (int v = 0; v < VW; ++v) {
+      const uint32_t w0 = r0[32 * v], w1 = r1[32 * v];
+      madd(aw[v], w0, one);
+      madd(aw[v], w1, one);
+      ah[v] += __byte_perm(w0, 0u, 0x4341) + __byte_perm(w1, 0u, 0x4341);
+    }
+    c += 2;
+  }
+  if (cnt & 1) {
+    const uint32_t* r0 = reinterpret_cast<const uint32_t*>(base + e[c]);
+#pragma unroll
+    for (int v = 0; v < VW; ++v) {
+      const uint32_t w0 = r0[32 * v];
+      madd(aw[v], w0, one);
+      ah[v] += __byte_perm(w0, 0u, 0x4341);
+    }
+  }
+}
+
+// Moves the sums one sample to the front: byte lane i of a word takes lane i + 1,
+// the last one lane 0 of the next word (lane + 1's; for lane 31 lane 0's of the
+// next 32 words). The last word of the tile gets no next one: each shift
+// spoils one more of its samples.
+template <int VW>
+__device__ __forceinline__ void wide1_shift(uint32_t (&aw)[VW], uint32_t (&ah)[VW], int lane) {
+  uint32_t nx[VW];
+#pragma unroll
+  for (int v = 0; v < VW; ++v) {
+    asm("mad.lo.u32 %0, %1, 0xFFFFFF00, %0;" : "+r"(aw[v]) : "r"(ah[v]));   // the even bytes' sums: aw - 256 ah
+    nx[v] = __shfl_sync(0xffffffffu, aw[v], (lane + 1) & 31);
+  }
+#pragma unroll
+  for (int v = 0; v < VW; ++v) {
+    const uint32_t n = v + 1 < VW && lane == 31 ? nx[v + 1 < VW ? v + 1 : v] : nx[v];
+    const uint32_t hi = __byte_perm(aw[v], n, 0x5432);
+    aw[v] = ah[v] + (hi << 8);
+    ah[v] = hi;
+  }
+}
+
+// Offset rows of the coarse DMs kk = pw, pw + kWide1Producers ... of an item:
+// {residue 3 | residue 2 << 16, residue 1 | residue 0 << 16} counts, then the
+// channels' byte offsets (of words) residue by residue, each part padded to four
+// entries. NCH: groups of 32 channels (m <= 32 NCH); KB coarse DMs' delays are
+// loaded at once. lead: the window start's residue mod 16; rb: bytes per channel.
+template <int NCH, int KB>
+__device__ __forceinline__ void wide1_rows(const int32_t* __restrict__ d1b, int nchan, int m, int n, int lead, int rb,
+                                            int tsu, uint32_t* __restrict__ tab, int pw, int lane) {
+  int d0[NCH];
+#pragma unroll
+  for (int g = 0; g < NCH; ++g) d0[g] = 32 * g + lane < m ? __ldg(d1b + 32 * g + lane) : 0;
+  const unsigned below = (1u << lane) - 1u;
+  for (int k0 = pw; k0 < n; k0 += kWide1Producers * KB) {
+    int x[KB][NCH];   // byte offsets of the channels' first samples; -1: no channel
+#pragma unroll
+    for (int i = 0; i < KB; ++i) {
+      const int32_t* d1k = d1b + (size_t)min(k0 + i * kWide1Producers, n - 1) * nchan;
+#pragma unroll
+      for (int g = 0; g < NCH; ++g) x[i][g] = 32 * g + lane < m ? __ldg(d1k + 32 * g + lane) : 0;
+    }
+#pragma unroll
+    for (int i = 0; i < KB; ++i) {
+      const int kk = k0 + i * kWide1Producers;
+      if (kk >= n) break;
+      uint32_t* row = tab + kk * tsu;
+      int cnt[4] = {0, 0, 0, 0};
+#pragma unroll
+      for (int g = 0; g < NCH; ++g) {
+        if (32 * g >= m) break;
+        x[i][g] = 32 * g + lane < m ? ((lead + d0[g]) & 15) + x[i][g] - d0[g] : -1;
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          cnt[r] += __popc(__ballot_sync(0xffffffffu, x[i][g] >= 0 && (x[i][g] & 3) == r));
+      }
+      int at[4];
+      at[3] = 4;
+      at[2] = at[3] + ((cnt[3] + 3) & ~3);
+      at[1] = at[2] + ((cnt[2] + 3) & ~3);
+      at[0] = at[1] + ((cnt[1] + 3) & ~3);
+      if (lane == 0)
+        *reinterpret_cast<uint2*>(row) =
+            make_uint2((uint32_t)cnt[3] | (uint32_t)cnt[2] << 16, (uint32_t)cnt[1] | (uint32_t)cnt[0] << 16);
+#pragma unroll
+      for (int g = 0; g < NCH; ++g) {
+        if (32 * g >= m) break;
+        int pos = 0;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const bool in = x[i][g] >= 0 && (x[i][g] & 3) == r;
+          const unsigned b = __ballot_sync(0xffffffffu, in);
+          if (in) pos = at[r] + __popc(b & below);
+          at[r] += __popc(b);
+        }
+        if (x[i][g] >= 0) row[pos] = (uint32_t)((32 * g + lane) * rb + (x[i][g] & ~3));
+      }
+    }
+  }
+}
+
+// What the roles of a block hand each other.
+struct Wide1Shared {
+  uint64_t full[kWide1MaxStages], empty[kWide1MaxStages];
+  Stage1Item desc[kWide1MaxStages];
+  int item[kWide1MaxStages];   // the stage's item; nitems or more: no more; -1: given up
+  int beam[kWide1MaxStages];   // whose arguments apply
+  int abort_flag;
+};
+
+// Persistent blocks take work items (sub-band s, coarse DMs [kb, ke), a tile of
+// 128 VW times from tau0) from a per-launch counter, in a batch the members'
+// items in turn (unit u of member j is item u - off[j] of its plan), through
+// `nst` shared-memory stages without block-wide barriers:
+//   * kWide1Producers warps bulk-copy (TMA) the channels' input windows, one
+//     byte per sample from 16-byte aligned ring positions (in pieces where a
+//     window wraps the ring's end), and write per coarse DM the channels' word
+//     offsets, sorted by the residue mod 4 of their byte offsets;
+//   * each consumer warp sums whole coarse DMs: kk = its number less a rotating
+//     base, + kWide1Consumers ..., so that work evens out over items.
+// An output word j of lane l holds the four sums of samples 4 (l + 32 j) .. + 3.
+// A channel whose window starts at byte offset o contributes the aligned words
+// from o / 4 on; the o % 4 samples by which they are early are made up for
+// once per residue: channels of residue 3 are summed first, the sums move
+// one sample to the front, residue 2 is added, and so on. So no delay needs a
+// rearranged copy, and each word feeds four outputs:
+//   sum w = sum(even bytes) + 256 * sum(odd bytes)   (mod 2^32)
+// with the odd bytes accumulated separately as 16-bit lanes, exact for up to
+// 257 channels. Consecutive outputs leave as one 8-byte store.
+// Used for sub-bands of more than 64 channels: k_stage1 rearranges an item's
+// windows into 32-bit words four times their size, which leaves such
+// sub-bands tiles of 512 or 256 outputs and few coarse DMs to share them; one
+// byte per sample lets them keep 512 outputs, 64 coarse DMs and a second item
+// in flight. 125 channels per sub-band (1000 channels, 76 coarse DMs, 20160
+// samples): 231 -> 102 us; 96 channels (937 DMs in groups of 2, 17408 samples):
+// 128 -> 103 us. Both are bound by shared memory (a byte per sample-add) and issue; at 64
+// channels k_stage1's longest tile fits and its rearranged words need fewer
+// instructions: 2.70 against 2.73 ms on the MeerKAT-L block, 14.5 against 16.2
+// us on 16 channels per sub-band.
+// Waits are bounded as in k_stage2_pipe; only one producer warp waits for free
+// stages, the others follow it through a named barrier.
+template <int VW, typename PT, typename Src, bool HALF = false>
+__global__ void __launch_bounds__(kWide1Warps * 32, 1)
+k_stage1_wide(const Src src, const int32_t* __restrict__ uoff, const int32_t* __restrict__ umem, int nmem, int nitems,
+         const Wide1Shape sp, uint32_t unit, int32_t* __restrict__ ictr) {
+  extern __shared__ __align__(16) uint8_t smem1[];
+  __shared__ __align__(16) Wide1Shared sh;
+  pdl_wait();
+  pdl_trigger();
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if ((int)blockIdx.x >= nitems) return;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < sp.nst; ++i) {
+      mbar_init(&sh.full[i], kWide1Producers);
+      mbar_init(&sh.empty[i], kWide1Consumers);
+    }
+    sh.abort_flag = 0;
+    fence_mbar_init();
+  }
+  __syncthreads();   // barriers initialised: the only block-wide barrier
+  volatile int* abort = &sh.abort_flag;
+  // a wait that gave up: the items the block leaves undone may be any member's
+  auto give_up = [&]() {
+    if (atomicExch(&sh.abort_flag, 1) != 0) return;
+    if constexpr (Src::kBatch) {
+      for (int j = 0; j < nmem; ++j) record_give_up(src.get(umem[j]));
+    } else {
+      record_give_up(src.get(0));
+    }
+  };
+  MemberCursor cur;
+  int st = 0;
+  uint32_t par = 0u;
+
+  if (warp >= kWide1Consumers) {
+    // ------------------------------------------------------------------ producers
+    const int pw = warp - kWide1Consumers, ptid = threadIdx.x - kWide1Consumers * 32;
+    int nextv = blockIdx.x;   // (producer 0, lane 0) the next item, asked for one ahead
+    uint32_t polls = 0u;
+    if constexpr (!Src::kBatch) polls = src.get(0).polls; else polls = src.get(umem[0]).polls;
+    int64_t q = 0;
+    bool end = false;
+    while (true) {
+      if (pw == 0) {
+        const bool ok = q < sp.nst || mbar_wait_or_abort(&sh.empty[st], par ^ 1u, polls, abort);
+        if (!ok) give_up();
+        if (lane == 0) {
+          sh.item[st] = ok ? nextv : -1;
+          if (ok && nextv < nitems) {
+            int lu = nextv;
+            if constexpr (Src::kBatch) {
+              cur.seek(uoff, umem, nmem, nextv);
+              lu -= cur.lo;
+              sh.beam[st] = cur.beam;
+            }
+            const BeamArgs a = src.get(cur.beam);
+            sh.desc[st] = a.items[lu];
+            mbar_expect_only(&sh.full[st], (uint32_t)(a.m * sp.rb));
+            nextv = (int)gridDim.x + atomicAdd(ictr, 1);
+          }
+        }
+      }
+      __syncwarp();
+      asm volatile("bar.sync 1, %0;" ::"n"(kWide1Producers * 32) : "memory");
+      const int v = sh.item[st];
+      if (v < 0) break;
+      if (v >= nitems) {
+        if (lane == 0) mbar_arrive(&sh.full[st]);
+        end = true;
+        break;
+      }
+      const BeamArgs a = src.get(Src::kBatch ? sh.beam[st] : 0);
+      const Stage1Item it = sh.desc[st];
+      const int m = a.m, n = it.ke - it.kb;
+      uint8_t* raw = smem1 + (size_t)st * sp.stage;
+      const int32_t* d1b = a.d1 + (size_t)it.kb * a.nchan + it.s * m;
+      fence_proxy_async();
+      for (int c = ptid; c < m; c += kWide1Producers * 32) {
+        const int R = (int)a.R;
+        int64_t p = a.start + it.tau0 + __ldg(d1b + c);
+        while (p >= R) p -= R;
+        const uint8_t* row = a.ring + (size_t)(it.s * m + c) * R;
+        int from = (int)p & ~15;
+        for (int done = 0; done < sp.rb;) {
+          const int len = min(sp.rb - done, R - from);
+          bulk_g2s(raw + (size_t)c * sp.rb + done, row + from, (uint32_t)len, &sh.full[st]);
+          done += len;
+          from = 0;
+        }
+      }
+      uint32_t* tab = reinterpret_cast<uint32_t*>(raw + (size_t)m * sp.rb);
+      const int lead = (int)((a.start + it.tau0) & 15);
+      if (m <= 128) wide1_rows<4, 2>(d1b, a.nchan, m, n, lead, sp.rb, sp.tsu, tab, pw, lane);
+      else wide1_rows<9, 1>(d1b, a.nchan, m, n, lead, sp.rb, sp.tsu, tab, pw, lane);
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sh.full[st]);
+      ++q;
+      if (++st == sp.nst) { st = 0; par ^= 1u; }
+    }
+    if (ptid == 0) {
+      // copies still in flight complete before the block's shared memory is released (the stage that
+      // took the end mark is past its last item's)
+      for (int64_t r = max((int64_t)0, q - sp.nst + (end ? 1 : 0)); r < q; ++r)
+        mbar_wait(&sh.full[(int)(r % sp.nst)], (uint32_t)((r / sp.nst) & 1), kMbarPolls);
+    }
+    return;
+  }
+
+  // ------------------------------------------------------------------ consumers
+  uint32_t polls = 0u;
+  if constexpr (!Src::kBatch) polls = src.get(0).polls; else polls = src.get(umem[0]).polls;
+  int base = 0;   // rotates with the coarse DMs seen
+  while (true) {
+    if (!mbar_wait_or_abort(&sh.full[st], par, polls, abort)) {
+      give_up();
+      return;
+    }
+    if (sh.item[st] >= nitems) return;
+    const BeamArgs a = src.get(Src::kBatch ? sh.beam[st] : 0);
+    const int s = sh.desc[st].s, kb = sh.desc[st].kb, tau0 = sh.desc[st].tau0, n = sh.desc[st].ke - kb;
+    const uint8_t* raw = smem1 + (size_t)st * sp.stage;
+    const uint8_t* S = raw + 4 * lane;
+    const uint32_t* tab = reinterpret_cast<const uint32_t*>(raw + (size_t)a.m * sp.rb);
+    const int off = HALF ? a.hoff[s] : 0;   // the sub-band's offset (half intermediates)
+    for (int kk = warp >= base ? warp - base : warp - base + kWide1Consumers; kk < n; kk += kWide1Consumers) {
+      const size_t prow = (size_t)(kb + kk) * a.nsub + s;
+      const int rel = tau0 - __ldg(a.abase + prow);   // used after the sums
+      const uint32_t* row = tab + kk * sp.tsu;
+      const uint2 h = *reinterpret_cast<const uint2*>(row);
+      const int c3 = (int)(h.x & 0xFFFFu), c2 = (int)(h.x >> 16), c1 = (int)(h.y & 0xFFFFu), c0 = (int)(h.y >> 16);
+      const uint32_t* e = row + 4;
+      uint32_t aw[VW], ah[VW];
+#pragma unroll
+      for (int v = 0; v < VW; ++v) aw[v] = ah[v] = 0u;
+      wide1_add<VW>(aw, ah, S, e, c3, unit);
+      wide1_shift<VW>(aw, ah, lane);
+      e += (c3 + 3) & ~3;
+      wide1_add<VW>(aw, ah, S, e, c2, unit);
+      wide1_shift<VW>(aw, ah, lane);
+      e += (c2 + 3) & ~3;
+      wide1_add<VW>(aw, ah, S, e, c1, unit);
+      wide1_shift<VW>(aw, ah, lane);
+      e += (c1 + 3) & ~3;
+      wide1_add<VW>(aw, ah, S, e, c0, unit);
+      PT* o = static_cast<PT*>(a.P) + prow * a.Pp + (rel + 4 * lane);   // rel and Pp are multiples of 16
+#pragma unroll
+      for (int v = 0; v < VW; ++v) {
+        const uint32_t lo = aw[v] - (ah[v] << 8);
+        const int t = rel + 4 * (lane + 32 * v);
+        if (t < 0 || t >= a.Pp || (v == VW - 1 && lane >= 28)) continue;   // (the tile's last 16 samples are the next tile's)
+        const PT v0 = stage1_store<PT, HALF>(lo & 0xFFFFu, off), v1 = stage1_store<PT, HALF>(ah[v] & 0xFFFFu, off);
+        const PT v2 = stage1_store<PT, HALF>(lo >> 16, off), v3 = stage1_store<PT, HALF>(ah[v] >> 16, off);
+        if constexpr (sizeof(PT) == 2)
+          *reinterpret_cast<uint2*>(o + 128 * v) =
+              make_uint2((uint32_t)v0 | (uint32_t)v1 << 16, (uint32_t)v2 | (uint32_t)v3 << 16);
+        else
+          *reinterpret_cast<int4*>(o + 128 * v) = make_int4(v0, v1, v2, v3);
+      }
+    }
+    base = (base + n) % kWide1Consumers;
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&sh.empty[st]);
+    if (++st == sp.nst) { st = 0; par ^= 1u; }
+  }
+}
+
+// ---------------------------------------------------------------------------
 // stage 2 (Sec. 2.3: de-disperse the sub-bands on the fine DM grid)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void warp_sum_stats(long long& s1, unsigned long long& s2) {

@@ -45,6 +45,28 @@ int64_t stage1_smem_bytes(int m, int q) {
 
 static int64_t floor_div(int64_t a, int64_t b) { return a >= 0 ? a / b : -((-a + b - 1) / b); }
 
+Wide1Shape wide1_shape(int m, int most) {
+  // in order of preference: long tiles (the shifts and the row bases are paid
+  // once per tile and coarse DM), then wide spreads and many coarse DMs (a
+  // window is staged once for them all)
+  static const int shapes[][3] = {{8, 240, 64}, {8, 240, 32}, {4, 240, 64}, {4, 240, 32}, {4, 112, 32}, {4, 48, 16},
+                                  {2, 240, 64}, {2, 240, 32}, {2, 112, 32}, {2, 48, 16}};
+  Wide1Shape r{};
+  for (const auto& s : shapes) {
+    if (s[0] > most) continue;
+    r.vw = s[0];
+    r.span = s[1];
+    r.nmax = s[2];
+    r.rb = (int)round_up(15 + r.span + 128 * r.vw, 16);
+    r.tsu = (int)round_up(m + 16, 8);
+    r.stage = m * r.rb + r.nmax * r.tsu * 4;
+    r.nst = std::min(kWide1MaxStages, (kSmemMax - 2048) / r.stage);
+    if (r.nst >= 2) return r;
+  }
+  r.nst = 0;
+  return r;
+}
+
 // Eq. 1 in samples: rnd(K DM (1/f^2 - 1/f_ref^2) / t_samp), rnd = llround.
 static int64_t delay_samples(double dm, double f, double f_ref, double tsamp) {
   const double v = kDispersion * dm * (1.0 / (f * f) - 1.0 / (f_ref * f_ref)) / tsamp;
@@ -354,47 +376,60 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
   while (q1 > 32 && stage1_smem_bytes(m, q1) > kSmemMax) q1 /= 2;
   if (stage1_smem_bytes(m, q1) > kSmemMax) { set_error("too many channels per sub-band for stage 1 (%d)", m); return TX_ERR_UNSUPPORTED; }
   p->q1 = q1;
-  p->span1_max = q1 - 16;
-  const int64_t tt1 = 4 * (int64_t)q1;
-  // every window start of an execute is (head - L) mod R with head a multiple
-  // of 64 plus a multiple of T, and R a multiple of 64
-  p->tab1_phase = (int32_t)((16 - p->L % 16) % 16);
-  const int TS1 = (m + 3) & ~3, SW1 = kStage1StagedWords(q1);
-  p->tab1.clear();
-  for (int s = 0; s < nsub; ++s) {
-    int kb = 0;
-    while (kb < nk) {
-      auto spread = [&](int k0, int k1) {  // max_c d1[k1-1][c] - d1[k0][c]
-        int32_t v = 0;
-        for (int c = s * m; c < (s + 1) * m; ++c)
-          v = std::max(v, p->d1[(size_t)(k1 - 1) * nchan + c] - p->d1[(size_t)k0 * nchan + c]);
-        return v;
-      };
-      int ke = kb + 1;
-      while (ke < nk && ke - kb < kStage1MaxCoarse && spread(kb, ke + 1) <= p->span1_max) ++ke;
-      // 16, 32 or 64 coarse DMs keep the 32 warps evenly busy (two, one or half a warp per DM)
-      if (ke - kb >= 32) ke = kb + (ke - kb) / 32 * 32;
-      else if (ke - kb >= 16) ke = kb + 16;
-      const int32_t span = spread(kb, ke);
-      int64_t lo = INT64_MAX, hi = 0;
-      for (int k = kb; k < ke; ++k) {
-        lo = std::min<int64_t>(lo, p->abase[(size_t)k * nsub + s]);
-        hi = std::max<int64_t>(hi, (int64_t)p->abase[(size_t)k * nsub + s] + p->Pp);
-      }
-      const int32_t toff = (int32_t)p->tab1.size();
-      for (int kk = 0; kk < ke - kb; ++kk)
-        for (int c = 0; c < TS1; ++c) {
-          if (c >= m) { p->tab1.push_back(0); continue; }
-          const int32_t d0 = p->d1[(size_t)kb * nchan + s * m + c];
-          p->tab1.push_back(c * SW1 + ((p->tab1_phase + d0) & 15) + p->d1[(size_t)(kb + kk) * nchan + s * m + c] - d0);
+  // the longest tile that fits is shorter than 1024 samples: the wide kernel
+  // (a shorter tile asked for is taken as asked)
+  p->s1w = wide1_shape(m, 8);
+  p->wide1 = q1 < 256 && stage1_smem_bytes(m, 2 * q1) > kSmemMax && p->s1w.nst >= 2;
+  do {
+    p->items1.clear();
+    p->tab1.clear();
+    p->span1_max = p->wide1 ? p->s1w.span : q1 - 16;
+    const int most1 = p->wide1 ? p->s1w.nmax : kStage1MaxCoarse;
+    const int64_t tt1 = p->wide1 ? kWide1TileStep(p->s1w.vw) : 4 * (int64_t)q1;
+    // every window start of an execute is (head - L) mod R with head a multiple
+    // of 64 plus a multiple of T, and R a multiple of 64
+    p->tab1_phase = (int32_t)((16 - p->L % 16) % 16);
+    const int TS1 = (m + 3) & ~3, SW1 = kStage1StagedWords(q1);
+    for (int s = 0; s < nsub; ++s) {
+      int kb = 0;
+      while (kb < nk) {
+        auto spread = [&](int k0, int k1) {  // max_c d1[k1-1][c] - d1[k0][c]
+          int32_t v = 0;
+          for (int c = s * m; c < (s + 1) * m; ++c)
+            v = std::max(v, p->d1[(size_t)(k1 - 1) * nchan + c] - p->d1[(size_t)k0 * nchan + c]);
+          return v;
+        };
+        int ke = kb + 1;
+        while (ke < nk && ke - kb < most1 && spread(kb, ke + 1) <= p->span1_max) ++ke;
+        // 16, 32 or 64 coarse DMs keep the 32 warps evenly busy (two, one or half a warp per DM)
+        // (the wide kernel evens its warps out over items)
+        if (!p->wide1 && ke - kb >= 32) ke = kb + (ke - kb) / 32 * 32;
+        else if (!p->wide1 && ke - kb >= 16) ke = kb + 16;
+        const int32_t span = spread(kb, ke);
+        int64_t lo = INT64_MAX, hi = 0;
+        for (int k = kb; k < ke; ++k) {
+          lo = std::min<int64_t>(lo, p->abase[(size_t)k * nsub + s]);
+          hi = std::max<int64_t>(hi, (int64_t)p->abase[(size_t)k * nsub + s] + p->Pp);
         }
-      for (int kk = 0; kk < ((ke - kb + 3) & ~3); ++kk)   // the coarse DMs' P-row bases
-        p->tab1.push_back(kk < ke - kb ? p->abase[(size_t)(kb + kk) * nsub + s] : 0);
-      for (int64_t t0 = floor_div(lo, tt1) * tt1; t0 < hi; t0 += tt1)
-        p->items1.push_back(Stage1Item{s, kb, ke, (int32_t)t0, span, toff, 0, 0});
-      kb = ke;
+        const int32_t toff = (int32_t)p->tab1.size();
+        for (int kk = 0; kk < ke - kb && !p->wide1; ++kk)
+          for (int c = 0; c < TS1; ++c) {
+            if (c >= m) { p->tab1.push_back(0); continue; }
+            const int32_t d0 = p->d1[(size_t)kb * nchan + s * m + c];
+            p->tab1.push_back(c * SW1 + ((p->tab1_phase + d0) & 15) + p->d1[(size_t)(kb + kk) * nchan + s * m + c] - d0);
+          }
+        for (int kk = 0; kk < ((ke - kb + 3) & ~3) && !p->wide1; ++kk)   // the coarse DMs' P-row bases
+          p->tab1.push_back(kk < ke - kb ? p->abase[(size_t)(kb + kk) * nsub + s] : 0);
+        for (int64_t t0 = floor_div(lo, tt1) * tt1; t0 < hi; t0 += tt1)
+          p->items1.push_back(Stage1Item{s, kb, ke, (int32_t)t0, span, toff, 0, 0});
+        kb = ke;
+      }
     }
-  }
+    // few items: shorter tiles of the wide kernel keep the SMs busy
+    const Wide1Shape next = wide1_shape(m, p->s1w.vw / 2);
+    if (!p->wide1 || p->items1.size() >= (size_t)kWide1MinItems || p->s1w.vw <= 2 || next.nst < 2) break;
+    p->s1w = next;
+  } while (true);
   // Time-major order: blocks working at the same time read overlapping input
   // windows of every sub-band, which keeps the ring's working set in L2.
   std::stable_sort(p->items1.begin(), p->items1.end(), [](const Stage1Item& a, const Stage1Item& b) {

@@ -28,6 +28,15 @@ constexpr int kStage1Warps = 32;
 // bytes rounded up to 16-byte chunks.
 constexpr int kStage1StagedWords(int q) { return 2 * q + 4; }
 constexpr int kStage1RawBytes(int q) { return (5 * q + 2 + 15) / 16 * 16; }
+// Sub-bands of more than 64 channels (those whose longest tile above is shorter
+// than 1024 samples): a coarse DM's tile is `vw` 32-bit words per lane of a
+// warp, four consecutive samples to a word. The last 16 of a tile's samples are
+// slack (see k_stage1_wide) and belong to the next tile.
+constexpr int kWide1Consumers = 28;    // consumer warps
+constexpr int kWide1Producers = 4;     // copying and table-building warps
+constexpr int kWide1Warps = kWide1Consumers + kWide1Producers;
+constexpr int kWide1MaxStages = 8;     // items in flight
+constexpr int kWide1TileStep(int vw) { return 128 * vw - 16; }
 constexpr int kSmemMax = 232448;       // opt-in dynamic shared memory per block (227 KB)
 
 // Polls of an mbarrier before a kernel gives up waiting for a bulk copy; each
@@ -122,6 +131,15 @@ struct DevicePlan {
 
 void set_error(const char* fmt, ...);
 int64_t stage1_smem_bytes(int m, int q);
+// The wide sub-bands' stage 1 for m channels, at most `most` words per lane: words per lane, the delay spread
+// and coarse DMs an item may have, bytes of a channel's window, words of a
+// coarse DM's offset row, bytes of a stage and how many fit.
+struct Wide1Shape {
+  int vw, span, nmax, rb, tsu, stage, nst;
+  int smem() const { return stage * nst; }
+};
+Wide1Shape wide1_shape(int m, int most);
+constexpr int kWide1MinItems = 2 * 152;   // items a plan keeps for a full GPU before shortening its tiles
 // Polling limit of the first wait for each bulk copy in the kernels launched
 // from now on (tx_set_wait_polls; kWaitPolls unless changed).
 uint32_t first_wait_polls();
@@ -160,6 +178,8 @@ struct tx_plan {
   int64_t head0 = 0;              // where a fresh beam's first block lands
   int32_t q1 = 256;               // stage-1 quarter length (words)
   int32_t span1_max = 256;        // staged delay spread limit of stage 1
+  int32_t wide1 = 0;              // stage 1 runs k_stage1_wide in the shape s1w
+  tx::Wide1Shape s1w{};
   int32_t span2_max = 0;          // max stage-2 delay spread within a group
   int32_t nw2 = 512;              // stage-2 tile words (2 * nw2 outputs)
   int32_t split2 = 2;             // stage-2 warps per fine DM (uint16 path)
