@@ -227,8 +227,9 @@ int build_batch(tx_batch* B, int64_t budget) {
       L.wave = wv;
       rc = add_members(L, mem, first, [&](int b) -> int64_t {
         const tx_plan* p = B->plans[b];
-        return p->layout == TX_LAYOUT_TF ? ((p->T + 63) / 64) * ((p->nchan + 63) / 64)
-                                         : (int64_t)p->nchan * ((p->T + 4095) / 4096);
+        const int64_t n = p->T + ingest_slack(p->T, B->beams[b]->compact);
+        return p->layout == TX_LAYOUT_TF ? ((n + 63) / 64) * ((p->nchan + 63) / 64)
+                                         : (int64_t)p->nchan * ((n + 4095) / 4096);
       });
       if (rc) return rc;
       L.threads = 256;

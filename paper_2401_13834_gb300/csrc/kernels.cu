@@ -191,15 +191,16 @@ int ingest(const tx_plan* p, const uint8_t* src, int64_t n, uint8_t* ring, int64
   pos = mod(pos, R);
   while (done < n) {
     const int64_t len = std::min(n - done, R - pos);
+    const int64_t span = len + pos % 16;   // on the ring's 16-byte grid
     if (p->layout == TX_LAYOUT_TF) {
-      const int vec = (p->nchan % 16 == 0) && (pos % 16 == 0) && (((uintptr_t)src & 15) == 0);
-      dim3 grid((unsigned)((len + 64 * kIngestTiles - 1) / (64 * kIngestTiles)), (unsigned)((p->nchan + 63) / 64));
-      TX_CUDA(launch_pdl(k_ingest_tf, grid, 256, 0, st, src, done, len, p->nchan, ring, R, pos, vec, zero));
+      dim3 grid((unsigned)((span + 64 * kIngestTiles - 1) / (64 * kIngestTiles)), (unsigned)((p->nchan + 63) / 64));
+      TX_CUDA(launch_pdl(k_ingest_tf, grid, 256, 0, st, src, done, len, p->nchan, ring, R, pos,
+                         tf_load_form(src, p->nchan), zero));
     } else {
-      const int vec = (n % 16 == 0) && (done % 16 == 0) && (len % 16 == 0) && (pos % 16 == 0) &&
-                      (((uintptr_t)src & 15) == 0);
-      dim3 grid((unsigned)std::min<int64_t>((len + 4095) / 4096, 64), (unsigned)p->nchan);
-      TX_CUDA(launch_pdl(k_ingest_ft, grid, 256, 0, st, src, n, done, len, ring, R, pos, vec, zero));
+      dim3 grid((unsigned)std::min<int64_t>((span + 4095) / 4096, 64), (unsigned)p->nchan);
+      const bool vec = (n | done | len | pos | (int64_t)(uintptr_t)src) % 16 == 0;
+      TX_CUDA(launch_pdl(vec ? k_ingest_ft<true> : k_ingest_ft<false>, grid, 256, 0, st, src, n, done, len, ring, R, pos,
+                         zero));
     }
     TX_CUDA(cudaGetLastError());
     done += len;
@@ -343,10 +344,10 @@ int32_t tx_beam_prime(const tx_plan* p, tx_beam* b, const uint8_t* d_tail, void*
     cudaStream_t st = (cudaStream_t)stream;
     uint8_t* t = b->tail + p->tail_pad;
     if (p->layout == TX_LAYOUT_TF) {
-      const int vec = (p->tail_pad % 16 == 0) && (p->nchan % 16 == 0) && (((uintptr_t)d_tail & 15) == 0);
-      dim3 grid((unsigned)((p->L + 64 * kIngestTiles - 1) / (64 * kIngestTiles)), (unsigned)((p->nchan + 63) / 64));
-      k_ingest_tf<<<grid, 256, 0, st>>>(d_tail, 0, p->L, p->nchan, b->tail, p->tail_pitch, p->tail_pad, vec,
-                                        nullptr);
+      dim3 grid((unsigned)((p->L + p->tail_pad + 64 * kIngestTiles - 1) / (64 * kIngestTiles)),
+                (unsigned)((p->nchan + 63) / 64));
+      k_ingest_tf<<<grid, 256, 0, st>>>(d_tail, 0, p->L, p->nchan, b->tail, p->tail_pitch, p->tail_pad,
+                                        tf_load_form(d_tail, p->nchan), nullptr);
       TX_CUDA(cudaGetLastError());
     } else {
       TX_CUDA(cudaMemcpy2DAsync(t, (size_t)p->tail_pitch, d_tail, (size_t)p->L, (size_t)p->L, (size_t)p->nchan,

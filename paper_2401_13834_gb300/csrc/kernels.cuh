@@ -34,6 +34,7 @@
 #include <utility>
 
 #include "device.cuh"
+#include "ingest.cuh"
 #include "tx_internal.h"
 
 namespace {
@@ -72,7 +73,7 @@ struct BeamArgs {
   int32_t tail_pad, tab1_phase;
   int32_t box_tile;              // boxcar outputs per unit (a multiple of kBoxTile)
   uint32_t polls;                // polling limit of the first wait for each bulk copy
-  int8_t layout, ingest_vec, running, output, compact, half, box_vec;
+  int8_t layout, ingest_ld, running, output, compact, half, box_vec;
 };
 // Two constant-memory slots of kArgSlotBeams of these fit the 64 KB bank.
 static_assert(sizeof(BeamArgs) <= 352, "BeamArgs grew");
@@ -141,82 +142,59 @@ __device__ __forceinline__ void madd_hi16(uint32_t& acc, uint32_t a) {
 // ---------------------------------------------------------------------------
 // Both ingest kernels also zero *zero (when given): the stage-1 item counter
 // of the execute, so that no launch of its own is spent on it.
-// Channel-major rows: ring[c][dst_off + i] = src[c][src_off + i], i < n.
-__global__ void k_ingest_ft(const uint8_t* __restrict__ src, int64_t src_pitch, int64_t src_off, int64_t n,
-                            uint8_t* __restrict__ ring, int64_t R, int64_t dst_off, int vec, int32_t* zero) {
+// Blocks land in the ring on the ring's own 16-byte grid: tiles and chunks
+// start at ring positions that are multiples of 16, whatever the block's length,
+// and only the block's first and last few samples take byte stores. (The
+// rows of a time-major block may start anywhere; those of a channel-major one
+// are read as aligned words and shifted.)
+
+// Channel-major rows: ring[c][dst_off + i] = src[c][src_off + i], i < n, 16
+// samples of the ring's grid per thread. VEC: whole aligned 16-byte groups on
+// both sides (a kernel of its own: with the other form's registers it ran at
+// 107 instead of 91 us on the 268 MB block).
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_ingest_ft(const uint8_t* __restrict__ src, int64_t src_pitch, int64_t src_off,
+                                                   int64_t n, uint8_t* __restrict__ ring, int64_t R, int64_t dst_off,
+                                                   int32_t* zero) {
   pdl_wait();
   pdl_trigger();
   if (zero && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *zero = 0;
   const int c = blockIdx.y;
-  const uint8_t* s = src + (int64_t)c * src_pitch + src_off;
+  const uint8_t* row = src + (int64_t)c * src_pitch + src_off;
   uint8_t* d = ring + (int64_t)c * R + dst_off;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  if (vec) {
-    const uint4* s4 = reinterpret_cast<const uint4*>(s);
+  if constexpr (VEC) {
+    const uint4* s4 = reinterpret_cast<const uint4*>(row);
     uint4* d4 = reinterpret_cast<uint4*>(d);
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n / 16; i += stride) d4[i] = s4[i];
   } else {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) d[i] = s[i];
+    const uint8_t* end = src + src_pitch * gridDim.y;
+    const int shift = (int)(dst_off & 15);
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; 16 * i - shift < n; i += stride) {
+      const int64_t t = 16 * i - shift;
+      store16(d + t, ft_chunk(src, end, row, t, n), t, n);
+    }
   }
 }
 
 constexpr int kIngestTiles = 4;
 
-// This thread's 16 bytes of the 64-time x 64-channel byte tile (times t0..,
-// channels c0..) of a time-major block [t][nchan]: time t0 + tid / 4,
-// channels c0 + 16 (tid % 4) ..; zero outside the block. 256 threads.
-__device__ __forceinline__ uint4 tf_tile_chunk(const uint8_t* __restrict__ src, int64_t t0, int64_t n, int c0,
-                                               int nchan, int vec) {
-  const int r = threadIdx.x >> 2, q = threadIdx.x & 3;
-  const int64_t t = t0 + r;
-  const int c = c0 + 16 * q;
-  uint4 v = make_uint4(0u, 0u, 0u, 0u);
-  if (t < n) {
-    const uint8_t* sp = src + t * nchan + c;
-    if (vec && c + 16 <= nchan) {
-      v = __ldg(reinterpret_cast<const uint4*>(sp));
-    } else {
-      uint32_t w[4] = {0u, 0u, 0u, 0u};
-      for (int i = 0; i < 16; ++i)
-        if (c + i < nchan) w[i >> 2] |= (uint32_t)sp[i] << (8 * (i & 3));
-      v = make_uint4(w[0], w[1], w[2], w[3]);
-    }
-  }
-  return v;
-}
-
-// Loads such a tile into tile[time][channel].
-__device__ __forceinline__ void tf_load_tile(uint8_t (*tile)[80], const uint8_t* __restrict__ src, int64_t t0,
-                                             int64_t n, int c0, int nchan, int vec) {
-  *reinterpret_cast<uint4*>(&tile[threadIdx.x >> 2][16 * (threadIdx.x & 3)]) =
-      tf_tile_chunk(src, t0, n, c0, nchan, vec);
-}
-
-// Column cc of a tile, times 16 pq .. 16 pq + 15, as four little-endian words.
-__device__ __forceinline__ void tf_column(const uint8_t (*tile)[80], int cc, int pq, uint32_t w[4]) {
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    w[i] = (uint32_t)tile[16 * pq + 4 * i][cc] | ((uint32_t)tile[16 * pq + 4 * i + 1][cc] << 8) |
-           ((uint32_t)tile[16 * pq + 4 * i + 2][cc] << 16) | ((uint32_t)tile[16 * pq + 4 * i + 3][cc] << 24);
-}
-
 // Time-major block rows [t][nchan], t in [t_off, t_off + n) -> ring[c][dst_off + t - t_off],
 // through 64-time x 64-channel byte tiles, kIngestTiles consecutive ones per
-// block (blockIdx.x: times 64 kIngestTiles blockIdx.x ..; blockIdx.y: channels
-// 64 blockIdx.y ..). vec: 16-byte loads and stores (nchan, dst_off and the
-// source all 16-byte aligned).
+// block (blockIdx.x: from time 64 kIngestTiles blockIdx.x less dst_off's
+// residue; blockIdx.y: channels 64 blockIdx.y ..). ld: see tf_load_form.
 __global__ void __launch_bounds__(256) k_ingest_tf(const uint8_t* __restrict__ src, int64_t t_off, int64_t n,
                                                    int nchan, uint8_t* __restrict__ ring, int64_t R,
-                                                   int64_t dst_off, int vec, int32_t* zero) {
+                                                   int64_t dst_off, int ld, int32_t* zero) {
   __shared__ __align__(16) uint8_t tiles[kIngestTiles][64][80];
   pdl_wait();
   pdl_trigger();
   if (zero && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *zero = 0;
-  const int c0 = blockIdx.y * 64;
+  const int c0 = blockIdx.y * 64, shift = (int)(dst_off & 15);
   uint4 vv[kIngestTiles];   // all of the block's loads in flight at once
 #pragma unroll
   for (int i = 0; i < kIngestTiles; ++i)
-    vv[i] = tf_tile_chunk(src + t_off * nchan, ((int64_t)blockIdx.x * kIngestTiles + i) * 64, n, c0, nchan, vec);
+    vv[i] = tf_tile_chunk(src + t_off * nchan, ((int64_t)blockIdx.x * kIngestTiles + i) * 64 - shift, n, c0, nchan, ld);
 #pragma unroll
   for (int i = 0; i < kIngestTiles; ++i)
     *reinterpret_cast<uint4*>(&tiles[i][threadIdx.x >> 2][16 * (threadIdx.x & 3)]) = vv[i];
@@ -226,17 +204,10 @@ __global__ void __launch_bounds__(256) k_ingest_tf(const uint8_t* __restrict__ s
   if (c >= nchan) return;
 #pragma unroll 1
   for (int i = 0; i < kIngestTiles; ++i) {
-    const int64_t t0 = ((int64_t)blockIdx.x * kIngestTiles + i) * 64;
+    const int64_t t = ((int64_t)blockIdx.x * kIngestTiles + i) * 64 - shift + 16 * pq;
     uint32_t w[4];
     tf_column(tiles[i], cc, pq, w);
-    const int64_t t = t0 + 16 * pq;
-    uint8_t* dp = ring + (int64_t)c * R + dst_off + t;
-    if (vec && t + 16 <= n) {
-      *reinterpret_cast<uint4*>(dp) = make_uint4(w[0], w[1], w[2], w[3]);
-    } else {
-      for (int j = 0; j < 16; ++j)
-        if (t + j < n) dp[j] = (uint8_t)(w[j >> 2] >> (8 * (j & 3)));
-    }
+    store16(ring + (int64_t)c * R + dst_off + t, make_uint4(w[0], w[1], w[2], w[3]), t, n);
   }
 }
 
@@ -244,7 +215,11 @@ __global__ void __launch_bounds__(256) k_ingest_tf(const uint8_t* __restrict__ s
 // block and write them into that beam's ring at ring position head + t
 // (mod R, R a multiple of 64, so an aligned 16-byte group never straddles the
 // wrap). Time-major tiles are 64 times x 64 channels; channel-major tiles are
-// 4096 samples of one channel.
+// 4096 samples of one channel; both start on the ring's 16-byte grid.
+// Samples a beam's tiles must cover beyond its block's for any head: none
+// where every block starts on that grid.
+__host__ __device__ __forceinline__ int ingest_slack(int64_t T, int compact) { return T % 16 != 0 && !compact ? 15 : 0; }
+
 template <typename Src>
 __global__ void __launch_bounds__(256) k_ingest_batch(const Src src, const int32_t* __restrict__ uoff,
                                                       const int32_t* __restrict__ umem, int nmem, int nunits) {
@@ -258,18 +233,19 @@ __global__ void __launch_bounds__(256) k_ingest_batch(const Src src, const int32
     const BeamArgs b = src.get(nxt.beam);
     if (b.layout != TX_LAYOUT_TF) return;
     const int lu = u - nxt.lo, nct = (b.nchan + 63) >> 6;
-    pre = tf_tile_chunk(b.block, (int64_t)(lu / nct) * 64, b.T, (lu % nct) * 64, b.nchan, b.ingest_vec);
+    pre = tf_tile_chunk(b.block, (int64_t)(lu / nct) * 64 - (b.head & 15), b.T, (lu % nct) * 64, b.nchan, b.ingest_ld);
   };
   if ((int)blockIdx.x < nunits) tf_fetch(blockIdx.x);
   for (int u = blockIdx.x; u < nunits; u += gridDim.x) {
     cur.seek(uoff, umem, nmem, u);
     const int lu = u - cur.lo;
     const BeamArgs a = src.get(cur.beam);
+    const int shift = (int)(a.head & 15);
     if (a.half && lu == 0)  // k_offsets accumulates into these next
       for (int i = threadIdx.x; i <= a.nsub; i += blockDim.x) a.hoff[i] = 0;
     if (a.layout == TX_LAYOUT_TF) {
       const int nct = (a.nchan + 63) >> 6;
-      const int64_t t0 = (int64_t)(lu / nct) * 64;
+      const int64_t t0 = (int64_t)(lu / nct) * 64 - shift;
       const int c0 = (lu % nct) * 64;
       __syncthreads();  // the previous tile's readers are done with `tile`
       *reinterpret_cast<uint4*>(&tile[threadIdx.x >> 2][16 * (threadIdx.x & 3)]) = pre;
@@ -283,37 +259,18 @@ __global__ void __launch_bounds__(256) k_ingest_batch(const Src src, const int32
         const int64_t t = t0 + 16 * pq;
         int64_t pos = a.head + t;
         if (pos >= a.R) pos -= a.R;
-        uint8_t* row = a.ring + (int64_t)c * a.R;
-        if (a.ingest_vec && t + 16 <= a.T) {
-          *reinterpret_cast<uint4*>(row + pos) = make_uint4(w[0], w[1], w[2], w[3]);
-        } else {
-          for (int i = 0; i < 16; ++i) {
-            if (t + i >= a.T) break;
-            int64_t pb = pos + i;
-            if (pb >= a.R) pb -= a.R;
-            row[pb] = (uint8_t)(w[i >> 2] >> (8 * (i & 3)));
-          }
-        }
+        store16(a.ring + (int64_t)c * a.R + pos, make_uint4(w[0], w[1], w[2], w[3]), t, a.T);
       }
     } else {
       if (u + (int)gridDim.x < nunits) tf_fetch(u + gridDim.x);
-      const int nchunk = (int)((a.T + 4095) >> 12);
+      const int nchunk = (int)((a.T + ingest_slack(a.T, a.compact) + 4095) >> 12);
       const int c = lu / nchunk;
-      const int64_t t = (int64_t)(lu - c * nchunk) * 4096 + 16 * threadIdx.x;
+      const int64_t t = (int64_t)(lu - c * nchunk) * 4096 + 16 * threadIdx.x - shift;
       if (t < a.T) {
-        const uint8_t* src = a.block + (int64_t)c * a.T;
-        uint8_t* row = a.ring + (int64_t)c * a.R;
         int64_t pos = a.head + t;
         if (pos >= a.R) pos -= a.R;
-        if (a.ingest_vec && t + 16 <= a.T) {
-          *reinterpret_cast<uint4*>(row + pos) = __ldg(reinterpret_cast<const uint4*>(src + t));
-        } else {
-          for (int i = 0; i < 16 && t + i < a.T; ++i) {
-            int64_t pb = pos + i;
-            if (pb >= a.R) pb -= a.R;
-            row[pb] = src[t + i];
-          }
-        }
+        store16(a.ring + (int64_t)c * a.R + pos,
+                ft_chunk(a.block, a.block + (int64_t)a.nchan * a.T, a.block + (int64_t)c * a.T, t, a.T), t, a.T);
       }
     }
   }
@@ -2377,8 +2334,7 @@ inline BeamArgs make_args(const tx_plan* p, const tx_beam* b, const uint8_t* blo
   a.nw = p->nw;
   a.wmax = p->wmax;
   a.layout = p->layout;
-  const bool al = ((uintptr_t)block & 15) == 0 && head % 16 == 0;
-  a.ingest_vec = p->layout == TX_LAYOUT_TF ? (al && p->nchan % 16 == 0) : (al && p->T % 16 == 0);
+  a.ingest_ld = (int8_t)tf_load_form(block, p->nchan);
   a.running = p->stats == TX_STATS_RUNNING;
   a.output = p->output;
   a.polls = first_wait_polls();
