@@ -710,7 +710,7 @@ def run_ours(args):
             phases[name] = entry
         dom = max(phase_ms, key=phase_ms.get)
         if plan.interm == "f32":
-            kernel_of = {"ingest": "k_norm_ingest", "stage1": "k_stage1_f32", "stage2": "k_stage2_pipe32",
+            kernel_of = {"ingest": "k_norm_ingest_tf", "stage1": "k_stage1_f32", "stage2": "k_stage2_pipe32",
                          "stats": "k_stats_f32", "boxcar": "k_boxcar_f32"}
         else:
             kernel_of = {"ingest": "k_ingest_tf", "stage1": "k_stage1", "stage2": "k_stage2_pipe" if plan.tile_split2

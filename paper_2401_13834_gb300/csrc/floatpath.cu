@@ -3,9 +3,9 @@
 // Eq. 5), for plans with a tx_norm mode.
 //
 // Per block of a beam:
-//   k_chan_sums     exact sums of x and x^2 per channel over the block's T new samples
+//   k_chan_sums_*   exact sums of x and x^2 per channel over the block's T new samples
 //   k_chan_weights  mu_c, sigma_c (population), weight w_c = 1/sigma_c or 1/sigma_c^2
-//   k_norm_ingest   x' = (float(x) - mu_c) * w_c into the beam's float32 circular buffer
+//   k_norm_ingest_* x' = (float(x) - mu_c) * w_c into the beam's float32 circular buffer
 //                   behind the carried tail (which keeps its own block's normalisation)
 //   k_stage1_f32    P[k][s][t] = sum_{c in s} x'[c][t + d1[k][c]]  (FP32, channels in order)
 //   k_stage2_pipe32 D[d][t]    = sum_s P[k(d)][s][t + d2[d][s]]     (FP32, sub-bands in order),
@@ -22,6 +22,7 @@
 #include <cstdint>
 
 #include "device.cuh"
+#include "ingest.cuh"
 #include "stage2_pipe32.cuh"
 #include "tx_internal.h"
 
@@ -39,51 +40,99 @@ using namespace tx;
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kSumChunk = 4096;   // samples per block of the channel sums
+constexpr int kSumBytes = 16384;  // bytes of a channel-major row per block of the channel sums
 
 // ---- channel statistics -----------------------------------------------------
 // S[c] = (sum x, sum x^2) over samples t < n of channel c; block in the plan's
 // layout (FT rows of `pitch` bytes, or TF rows of nchan bytes). Atomic integer
-// adds: exact and order-free.
-__global__ void __launch_bounds__(kThreads) k_chan_sums(const uint8_t* __restrict__ blk, int layout, int nchan,
-                                                         int64_t n, int64_t pitch, unsigned long long* __restrict__ S) {
-  const int64_t t0 = (int64_t)blockIdx.x * kSumChunk;
-  const int64_t t1 = min(n, t0 + kSumChunk);
-  unsigned long long s1 = 0, s2 = 0;
-  if (layout == TX_LAYOUT_FT) {
-    const int c = blockIdx.y;
-    const uint8_t* row = blk + (int64_t)c * pitch;
-    for (int64_t t = t0 + threadIdx.x; t < t1; t += kThreads) {
-      const unsigned x = row[t];
-      s1 += x;
-      s2 += x * x;
-    }
-    __shared__ unsigned long long r1[kThreads / 32], r2[kThreads / 32];
+// adds: exact and order-free. Both read four samples of a channel per
+// instruction (dp4a): with one byte per load and one per store of the samples, a
+// MeerKAT-L block took 0.83 ms to normalise (now 0.31), and 320 channels x 14336
+// samples 0.29 ms on the eight SMs that summed them (now 0.02).
+//
+// Channel-major: one block per (row, kSumBytes bytes of it).
+__global__ void __launch_bounds__(kThreads) k_chan_sums_ft(const uint8_t* __restrict__ blk, int64_t n, int64_t pitch,
+                                                            unsigned long long* __restrict__ S) {
+  pdl_wait();
+  pdl_trigger();
+  const int c = blockIdx.y;
+  const uint8_t* row = blk + (int64_t)c * pitch;
+  const uint8_t* end = blk + (int64_t)gridDim.y * pitch;
+  const int64_t t0 = (int64_t)blockIdx.x * kSumBytes, t1 = min(n, t0 + kSumBytes);
+  unsigned s1 = 0, s2 = 0;   // at most 64 samples a thread
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
-    if ((threadIdx.x & 31) == 0) { r1[threadIdx.x >> 5] = s1; r2[threadIdx.x >> 5] = s2; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      unsigned long long a = 0, b = 0;
-      for (int w = 0; w < kThreads / 32; ++w) { a += r1[w]; b += r2[w]; }
-      atomicAdd(S + 2 * c, a);
-      atomicAdd(S + 2 * c + 1, b);
-    }
-  } else {
-    // one channel per thread, consecutive threads on consecutive channels
-    const int c = blockIdx.y * kThreads + threadIdx.x;
-    if (c >= nchan) return;
-    for (int64_t t = t0; t < t1; ++t) {
-      const unsigned x = blk[t * nchan + c];
-      s1 += x;
-      s2 += x * x;
-    }
-    atomicAdd(S + 2 * c, s1);
-    atomicAdd(S + 2 * c + 1, s2);
+  for (int i = 0; i < kSumBytes / 16 / kThreads; ++i) {
+    const int64_t t = t0 + 16 * (threadIdx.x + i * kThreads);
+    if (t >= t1) break;
+    const uint4 v = ft_chunk(blk, end, row, t, t1);
+    s1 = __dp4a(v.x, 0x01010101u, __dp4a(v.y, 0x01010101u, __dp4a(v.z, 0x01010101u, __dp4a(v.w, 0x01010101u, s1))));
+    s2 = __dp4a(v.x, v.x, __dp4a(v.y, v.y, __dp4a(v.z, v.z, __dp4a(v.w, v.w, s2))));
   }
+  __shared__ unsigned r1[kThreads / 32], r2[kThreads / 32];
+  s1 = __reduce_add_sync(0xffffffffu, s1);
+  s2 = __reduce_add_sync(0xffffffffu, s2);
+  if ((threadIdx.x & 31) == 0) { r1[threadIdx.x >> 5] = s1; r2[threadIdx.x >> 5] = s2; }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long a = 0, b = 0;
+    for (int w = 0; w < kThreads / 32; ++w) { a += r1[w]; b += r2[w]; }
+    atomicAdd(S + 2 * c, a);
+    atomicAdd(S + 2 * c + 1, b);
+  }
+}
+
+// Time-major: blocks of 256 channels x `chunk` times (a multiple of 16, at most
+// kSumBytes). Thread q + 64 p takes channels 4 q .. 4 q + 3 at times 4 p .. 4 p +
+// 3 of every 16; four rows' words are transposed to a word per channel.
+__global__ void __launch_bounds__(kThreads) k_chan_sums_tf(const uint8_t* __restrict__ blk, int nchan, int64_t n,
+                                                            int chunk, int words, unsigned long long* __restrict__ S) {
+  __shared__ unsigned r1[4][kThreads], r2[4][kThreads];
+  pdl_wait();
+  pdl_trigger();
+  const int q = threadIdx.x & 63, p = threadIdx.x >> 6;
+  const int c = blockIdx.y * 256 + 4 * q;
+  const int64_t t0 = (int64_t)blockIdx.x * chunk, t1 = min(n, t0 + chunk);
+  unsigned s1[4] = {0u, 0u, 0u, 0u}, s2[4] = {0u, 0u, 0u, 0u};
+#pragma unroll 2
+  for (int64_t t = t0 + 4 * p; t < t1; t += 16) {
+    uint32_t w[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      w[i] = 0u;
+      if (t + i < t1) {
+        const uint8_t* s = blk + (t + i) * nchan + c;
+        if (words) {
+          if (c < nchan) w[i] = __ldg(reinterpret_cast<const uint32_t*>(s));
+        } else {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            if (c + k < nchan) w[i] |= (uint32_t)s[k] << (8 * k);
+        }
+      }
+    }
+    const uint32_t a0 = __byte_perm(w[0], w[1], 0x5140), a1 = __byte_perm(w[0], w[1], 0x7362);
+    const uint32_t b0 = __byte_perm(w[2], w[3], 0x5140), b1 = __byte_perm(w[2], w[3], 0x7362);
+    const uint32_t x[4] = {__byte_perm(a0, b0, 0x5410), __byte_perm(a0, b0, 0x7632), __byte_perm(a1, b1, 0x5410),
+                           __byte_perm(a1, b1, 0x7632)};
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      s1[k] = __dp4a(x[k], 0x01010101u, s1[k]);
+      s2[k] = __dp4a(x[k], x[k], s2[k]);
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    r1[p][4 * q + k] = s1[k];
+    r2[p][4 * q + k] = s2[k];
+  }
+  __syncthreads();
+  const int ch = blockIdx.y * 256 + threadIdx.x;
+  if (ch >= nchan) return;
+  unsigned long long a = 0, b = 0;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) { a += r1[i][threadIdx.x]; b += r2[i][threadIdx.x]; }
+  atomicAdd(S + 2 * ch, a);
+  atomicAdd(S + 2 * ch + 1, b);
 }
 
 // (mu_c, w_c) as floats from the exact sums over n samples: mu = S1 / n,
@@ -92,6 +141,8 @@ __global__ void __launch_bounds__(kThreads) k_chan_sums(const uint8_t* __restric
 // variance), 0 when sigma = 0.
 __global__ void k_chan_weights(const unsigned long long* __restrict__ S, int nchan, int64_t n, int norm,
                                float2* __restrict__ muw) {
+  pdl_wait();
+  pdl_trigger();
   const int c = blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= nchan) return;
   const unsigned long long s1 = S[2 * c], s2 = S[2 * c + 1];
@@ -108,40 +159,88 @@ __device__ __forceinline__ float norm_sample(unsigned x, float2 mw) {
   return __fmul_rn(__fsub_rn((float)x, mw.x), mw.y);
 }
 
-// x' of samples t < n into ring[c][(pos0 + t) mod R]. FT: one channel row per
-// blockIdx.y; TF: 64-time x 64-channel byte tiles transposed through shared memory.
-__global__ void __launch_bounds__(kThreads) k_norm_ingest(const uint8_t* __restrict__ src, int layout, int nchan,
-                                                           int64_t n, int64_t pitch, float* __restrict__ ring, int64_t R,
-                                                           int64_t pos0, const float2* __restrict__ muw) {
-  if (layout == TX_LAYOUT_FT) {
-    const int c = blockIdx.y;
-    const float2 mw = muw[c];
-    const uint8_t* row = src + (int64_t)c * pitch;
-    float* out = ring + (int64_t)c * R;
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += (int64_t)gridDim.x * blockDim.x) {
-      int64_t p = pos0 + t;
-      if (p >= R) p -= R;
-      out[p] = norm_sample(row[t], mw);
-    }
-    return;
+// x' of samples t < n into ring[c][(pos0 + t) mod R], four samples of the ring's
+// 16-byte grid per store (R is a multiple of 64, so none straddles the wrap).
+// d: the position of sample t, a multiple of 4.
+__device__ __forceinline__ void norm_store4(float* __restrict__ row, int64_t R, int64_t pos, uint32_t x, int64_t t,
+                                            int64_t n, float2 mw) {
+  if (pos >= R) pos -= R;
+  const float v[4] = {norm_sample(x & 255u, mw), norm_sample((x >> 8) & 255u, mw), norm_sample((x >> 16) & 255u, mw),
+                      norm_sample(x >> 24, mw)};
+  if (t >= 0 && t + 4 <= n) {
+    *reinterpret_cast<float4*>(row + pos) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (t + i >= 0 && t + i < n) row[pos + i] = v[i];
   }
-  __shared__ uint8_t tile[64][65];
-  const int64_t t0 = (int64_t)blockIdx.x * 64;
+}
+
+// Channel-major rows, one per blockIdx.y.
+__global__ void __launch_bounds__(kThreads) k_norm_ingest_ft(const uint8_t* __restrict__ src, int64_t n, int64_t pitch,
+                                                              float* __restrict__ ring, int64_t R, int64_t pos0,
+                                                              const float2* __restrict__ muw) {
+  pdl_wait();
+  pdl_trigger();
+  const int c = blockIdx.y, shift = (int)(pos0 & 3);
+  const float2 mw = muw[c];
+  const uint8_t* row = src + (int64_t)c * pitch;
+  float* out = ring + (int64_t)c * R;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; 4 * i - shift < n; i += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t t = 4 * i - shift;
+    uint32_t x = 0u;
+    if (t >= 0 && t + 4 <= n && ((uintptr_t)(row + t) & 3) == 0) {
+      x = __ldg(reinterpret_cast<const uint32_t*>(row + t));
+    } else {
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (t + k >= 0 && t + k < n) x |= (uint32_t)__ldg(row + t + k) << (8 * k);
+    }
+    norm_store4(out, R, pos0 + t, x, t, n, mw);
+  }
+}
+
+// Time-major blocks, kNormTiles 64-time x 64-channel byte tiles per block (all
+// loads in flight first) through shared memory, 16 lanes to a channel's 64
+// times. ld: see tf_load_form.
+constexpr int kNormTiles = 2;
+__global__ void __launch_bounds__(kThreads) k_norm_ingest_tf(const uint8_t* __restrict__ src, int nchan, int64_t n,
+                                                              float* __restrict__ ring, int64_t R, int64_t pos0, int ld,
+                                                              const float2* __restrict__ muw) {
+  __shared__ uint32_t tile[kNormTiles][64][17];   // a time's 64 channels, padded by a word
+  pdl_wait();
+  pdl_trigger();
   const int c0 = blockIdx.y * 64;
-  for (int i = threadIdx.x; i < 64 * 64; i += kThreads) {
-    const int tt = i >> 6, cc = i & 63;
-    const int64_t t = t0 + tt;
-    tile[tt][cc] = (t < n && c0 + cc < nchan) ? src[t * nchan + c0 + cc] : 0;
+  const int64_t t0 = (int64_t)blockIdx.x * kNormTiles * 64 - (pos0 & 3);
+  uint4 v[kNormTiles];
+#pragma unroll
+  for (int i = 0; i < kNormTiles; ++i) v[i] = tf_tile_chunk(src, t0 + 64 * i, n, c0, nchan, ld);
+#pragma unroll
+  for (int i = 0; i < kNormTiles; ++i) {
+    uint32_t* w = &tile[i][threadIdx.x >> 2][4 * (threadIdx.x & 3)];
+    w[0] = v[i].x;
+    w[1] = v[i].y;
+    w[2] = v[i].z;
+    w[3] = v[i].w;
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < 64 * 64; i += kThreads) {
-    const int cc = i >> 6, tt = i & 63;          // consecutive threads: consecutive times of one channel
-    const int c = c0 + cc;
-    const int64_t t = t0 + tt;
-    if (c >= nchan || t >= n) continue;
-    int64_t p = pos0 + t;
-    if (p >= R) p -= R;
-    ring[(int64_t)c * R + p] = norm_sample(tile[tt][cc], muw[c]);
+  const int l = threadIdx.x & 15;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const int cc = (threadIdx.x >> 4) + 16 * k, c = c0 + cc;
+    if (c >= nchan) break;
+    const float2 mw = muw[c];
+    float* row = ring + (int64_t)c * R;
+#pragma unroll
+    for (int i = 0; i < kNormTiles; ++i) {
+      const int64_t t = t0 + 64 * i + 4 * l;
+      if (t >= n) break;
+      uint32_t x = 0u;
+#pragma unroll
+      for (int j = 0; j < 4; ++j)
+        x |= (uint32_t)reinterpret_cast<const uint8_t*>(tile[i][4 * l + j])[cc] << (8 * j);
+      norm_store4(row, R, pos0 + t, x, t, n, mw);
+    }
   }
 }
 
@@ -514,23 +613,28 @@ int normalise_into(const tx_plan* p, const uint8_t* src, int64_t n, int64_t pitc
                    unsigned long long* S, float2* muw, cudaStream_t st) {
   if (n <= 0) return TX_OK;
   TX_CUDA(cudaMemsetAsync(S, 0, (size_t)p->nchan * 16, st));
-  const unsigned nchunk = (unsigned)((n + kSumChunk - 1) / kSumChunk);
-  if (p->layout == TX_LAYOUT_FT)
-    k_chan_sums<<<dim3(nchunk, (unsigned)p->nchan), kThreads, 0, st>>>(src, p->layout, p->nchan, n, pitch, S);
-  else
-    k_chan_sums<<<dim3(nchunk, (unsigned)((p->nchan + kThreads - 1) / kThreads)), kThreads, 0, st>>>(
-        src, p->layout, p->nchan, n, pitch, S);
-  TX_CUDA(cudaGetLastError());
-  k_chan_weights<<<(p->nchan + 127) / 128, 128, 0, st>>>(S, p->nchan, n, p->norm, muw);
-  TX_CUDA(cudaGetLastError());
+  const int ld = tf_load_form(src, p->nchan);
+  if (p->layout == TX_LAYOUT_FT) {
+    TX_CUDA(launch_pdl(k_chan_sums_ft, dim3((unsigned)((n + kSumBytes - 1) / kSumBytes), (unsigned)p->nchan),
+                       dim3(kThreads), 0, st, src, n, pitch, S));
+  } else {
+    // about eight blocks per SM over the channel groups and times
+    const int64_t groups = (p->nchan + 255) / 256, want = std::max<int64_t>(8 * p->dev.num_sms / groups, 1);
+    const int chunk = (int)std::min<int64_t>(kSumBytes, std::max<int64_t>(64, ((n + want - 1) / want + 15) / 16 * 16));
+    TX_CUDA(launch_pdl(k_chan_sums_tf, dim3((unsigned)((n + chunk - 1) / chunk), (unsigned)groups), dim3(kThreads), 0, st,
+                       src, p->nchan, n, chunk, (int)(ld > 0), S));
+  }
+  TX_CUDA(launch_pdl(k_chan_weights, dim3((p->nchan + 127) / 128), dim3(128), 0, st, S, p->nchan, n, p->norm, muw));
   pos = mod(pos, p->R);
+  const int64_t span = n + pos % 4;   // on the ring's 16-byte grid
   if (p->layout == TX_LAYOUT_FT)
-    k_norm_ingest<<<dim3((unsigned)std::min<int64_t>((n + kThreads - 1) / kThreads, 64), (unsigned)p->nchan), kThreads,
-                    0, st>>>(src, p->layout, p->nchan, n, pitch, ring, p->R, pos, muw);
+    TX_CUDA(launch_pdl(k_norm_ingest_ft, dim3((unsigned)std::min<int64_t>((span + 4 * kThreads - 1) / (4 * kThreads), 64),
+                                              (unsigned)p->nchan),
+                       dim3(kThreads), 0, st, src, n, pitch, ring, p->R, pos, muw));
   else
-    k_norm_ingest<<<dim3((unsigned)((n + 63) / 64), (unsigned)((p->nchan + 63) / 64)), kThreads, 0, st>>>(
-        src, p->layout, p->nchan, n, pitch, ring, p->R, pos, muw);
-  TX_CUDA(cudaGetLastError());
+    TX_CUDA(launch_pdl(k_norm_ingest_tf, dim3((unsigned)((span + 64 * kNormTiles - 1) / (64 * kNormTiles)),
+                                              (unsigned)((p->nchan + 63) / 64)),
+                       dim3(kThreads), 0, st, src, p->nchan, n, ring, p->R, pos, ld, muw));
   return TX_OK;
 }
 
