@@ -566,38 +566,60 @@ __global__ void __launch_bounds__(kThreads) k_boxcar_f32(const float* __restrict
     comp_add(s, c, v);
   }
   __syncthreads();
-  for (int i = threadIdx.x; i < n; i += kThreads) {
-    const float2 c0 = H[i];
-    float best = -INFINITY;
-    int bw = 0;
-    for (int w = 0; w < nw; ++w) {
-      const float2 c1 = H[i + sW[w]];
-      const float B = __fadd_rn(__fsub_rn(__fsub_rn(c1.x, c0.x), sMh[w]), __fsub_rn(__fsub_rn(c1.y, c0.y), sMl[w]));
-      const float snr = __fmul_rn(B, sInv[w]);
-      if (mode == TX_OUT_CUBE) outf[((size_t)d * nw + w) * T + t0 + i] = snr;
-      if (snr > best) { best = snr; bw = w; }
+  // outputs tid + 256 r, RR at once: a width's constants are read from shared
+  // memory once for them (the MeerKAT-L plane: 1.87 -> 1.52 ms)
+  constexpr int RR = 8;
+  for (int i0 = threadIdx.x; i0 - (int)threadIdx.x < n; i0 += RR * kThreads) {
+    float2 c0[RR];
+    float best[RR];
+    int bw[RR];
+#pragma unroll
+    for (int r = 0; r < RR; ++r) {
+      const int i = i0 + r * kThreads;
+      c0[r] = i < n ? H[i] : make_float2(0.f, 0.f);
+      best[r] = -INFINITY;
+      bw[r] = 0;
     }
-    if (mode == TX_OUT_PLANE) {
-      outf[(size_t)d * T + t0 + i] = best;
-      outw[(size_t)d * T + t0 + i] = (uint8_t)bw;
-    } else if (mode == TX_OUT_CANDS) {
-      const bool hit = best >= gamma;
-      const unsigned act = __activemask();
-      const unsigned hits = __ballot_sync(act, hit);
-      if (hits) {
+#pragma unroll 1
+    for (int w = 0; w < nw; ++w) {
+      const float2* Hw = H + i0 + sW[w];
+      const float mh = sMh[w], ml = sMl[w], inv = sInv[w];
+      float* o = outf + ((size_t)d * nw + w) * T + t0 + i0;   // cube
+#pragma unroll
+      for (int r = 0; r < RR; ++r) {
+        if (i0 + r * kThreads >= n) break;
+        const float2 c1 = Hw[r * kThreads];
+        const float B = __fadd_rn(__fsub_rn(__fsub_rn(c1.x, c0[r].x), mh), __fsub_rn(__fsub_rn(c1.y, c0[r].y), ml));
+        const float snr = __fmul_rn(B, inv);
+        if (mode == TX_OUT_CUBE) o[r * kThreads] = snr;
+        else if (snr > best[r]) { best[r] = snr; bw[r] = w; }
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < RR; ++r) {
+      const int i = i0 + r * kThreads;
+      if (mode == TX_OUT_PLANE) {
+        if (i < n) {
+          outf[(size_t)d * T + t0 + i] = best[r];
+          outw[(size_t)d * T + t0 + i] = (uint8_t)bw[r];
+        }
+      } else if (mode == TX_OUT_CANDS) {
+        const bool hit = i < n && best[r] >= gamma;
+        const unsigned hits = __ballot_sync(0xffffffffu, hit);
+        if (!hits) continue;
         const int leader = __ffs(hits) - 1;
         unsigned long long base = 0;
         if (lane == leader) base = atomicAdd(ncand, (unsigned long long)__popc(hits));
-        base = __shfl_sync(act, base, leader);
+        base = __shfl_sync(0xffffffffu, base, leader);
         if (hit) {
           const unsigned long long idx = base + __popc(hits & ((1u << lane) - 1u));
           if (idx < (unsigned long long)max_cands) {
-            tx_cand r;
-            r.dm_index = d;
-            r.t = (int32_t)(t0 + i);
-            r.w_index = bw;
-            r.snr = best;
-            cands[idx] = r;
+            tx_cand rec;
+            rec.dm_index = d;
+            rec.t = (int32_t)(t0 + i);
+            rec.w_index = bw[r];
+            rec.snr = best[r];
+            cands[idx] = rec;
           }
         }
       }
