@@ -742,10 +742,22 @@ int32_t tx_downsample(const uint8_t* d_in, int32_t layout, int32_t nchan, int64_
   int dev = 0, nsm = 0;
   TX_CUDA(cudaGetDevice(&dev));
   TX_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-  const int vec = layout == TX_LAYOUT_TF && nchan % 4 == 0 && ((uintptr_t)d_in & 3) == 0 && ((uintptr_t)d_out & 3) == 0;
-  const int64_t work = (nsamp / factor) * (vec ? nchan / 4 : nchan);
-  const int grid = (int)std::min<int64_t>((work + 255) / 256, (int64_t)std::max(nsm, 1) * 16);
-  k_downsample<<<std::max(grid, 1), 256, 0, (cudaStream_t)stream>>>(d_in, layout, nchan, nsamp, factor, vec, d_out);
+  int sh = 0;
+  while ((1 << sh) < factor) ++sh;
+  const int mode = downsample_mode(d_in, d_out, layout, nchan, nsamp, sh);
+  const int64_t outs = (nsamp >> sh) * nchan;
+  const int64_t work = mode == 3 ? outs / 16 : mode == 2 ? outs / 4 : mode == 1 && sh == 1 ? outs / 2 : outs;
+  const int grid = std::max(1, (int)std::min<int64_t>((work + 255) / 256, (int64_t)std::max(nsm, 1) * 16));
+#define TX_DS(M, U) k_downsample<M, U><<<grid, 256, 0, (cudaStream_t)stream>>>(d_in, layout, nchan, nsamp, sh, d_out)
+#define TX_DSU(M) (sh == 0 ? (TX_DS(M, 1)) : sh == 1 ? (TX_DS(M, 2)) : sh == 2 ? (TX_DS(M, 4)) : (TX_DS(M, 8)))
+  switch (mode) {
+    case 3: TX_DSU(3); break;
+    case 2: TX_DSU(2); break;
+    case 1: TX_DS(1, 1); break;
+    default: TX_DS(0, 1); break;
+  }
+#undef TX_DSU
+#undef TX_DS
   TX_CUDA(cudaGetLastError());
   return TX_OK;
 }

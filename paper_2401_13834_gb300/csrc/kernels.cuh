@@ -389,53 +389,98 @@ __global__ void __launch_bounds__(256) k_offsets(const Src src, const int32_t* _
 // De-dispersion plans (Sec. 2.3, last paragraph): the block averaged over f
 // consecutive samples per channel, rounded half up, so it stays uint8:
 //   out[t'] = (sum_{i<f} in[f t' + i] + f / 2) / f,  t' < n / f.
-// Time-major blocks [t][nchan] are read four channels per 32-bit word when
-// nchan is a multiple of four (vec), byte by byte otherwise; channel-major
-// blocks [nchan][n] one output per thread.
+// f = 1 << sh. The sums of four bytes ride in two words of 16-bit lanes for f up
+// to 256. Bound by the block's bytes; MODE is the widest access that the block's
+// shape and addresses allow (downsample_mode): with four bytes per load (one on
+// channel-major blocks) and a division per output the 268 MB MeerKAT-L block took 571
+// us (channel-major 1306) at f = 2, 4, 8, 16 and 32 together, now 261 (389).
+//   3: time-major, 16 channels per load;  2: time-major, 4 channels;
+//   1: channel-major, words of a row (four samples, f >= 2);
+//   0: either, byte by byte.
+template <int MODE, int U>
 __global__ void __launch_bounds__(256) k_downsample(const uint8_t* __restrict__ in, int layout, int nchan, int64_t n,
-                                                    int f, int vec, uint8_t* __restrict__ out) {
-  const int64_t nout = n / f;
+                                                    int sh, uint8_t* __restrict__ out) {
+  const int f = 1 << sh;
+  const int64_t nout = n >> sh;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+  const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const uint32_t half = (uint32_t)(f >> 1);
-  if (layout == TX_LAYOUT_TF && vec) {
-    const int nw = nchan >> 2;
-    const int64_t total = nout * nw;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-      const int64_t t = i / nw;
-      const int w = (int)(i - t * nw);
-      const uint32_t* src = reinterpret_cast<const uint32_t*>(in + t * f * nchan) + w;
-      uint32_t s0 = 0, s1 = 0, s2 = 0, s3 = 0;
-      for (int k = 0; k < f; ++k) {
-        const uint32_t v = __ldg(src + (int64_t)k * nw);
-        s0 += v & 0xFFu;
-        s1 += (v >> 8) & 0xFFu;
-        s2 += (v >> 16) & 0xFFu;
-        s3 += v >> 24;
+  if constexpr (MODE >= 2) {
+    constexpr int W = MODE == 3 ? 4 : 1;   // words per load
+    const int per = nchan / (4 * W);
+    const uint32_t hh = half * 0x10001u;
+    for (int64_t i = first; i < nout * per; i += stride) {
+      const int64_t t = i / per;
+      const int64_t at = (t << sh) * nchan + (i - t * per) * (4 * W);
+      uint32_t lo[W], hi[W];
+#pragma unroll
+      for (int w = 0; w < W; ++w) lo[w] = hi[w] = 0u;
+      for (int k = 0; k < f; k += U) {
+        uint32_t v[U][W];   // U rows' loads in flight
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const uint8_t* p = in + at + (int64_t)(k + u) * nchan;
+          if constexpr (W == 4) {
+            const uint4 x = __ldg(reinterpret_cast<const uint4*>(p));
+            v[u][0] = x.x; v[u][1] = x.y; v[u][2] = x.z; v[u][3] = x.w;
+          } else {
+            v[u][0] = __ldg(reinterpret_cast<const uint32_t*>(p));
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int w = 0; w < W; ++w) {
+            lo[w] += v[u][w] & 0x00FF00FFu;
+            hi[w] += (v[u][w] >> 8) & 0x00FF00FFu;
+          }
       }
-      const uint32_t o = ((s0 + half) / f) | (((s1 + half) / f) << 8) | (((s2 + half) / f) << 16) |
-                         (((s3 + half) / f) << 24);
-      reinterpret_cast<uint32_t*>(out + t * nchan)[w] = o;
+      uint32_t o[W];
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        o[w] = (((lo[w] + hh) >> sh) & 0x00FF00FFu) | ((((hi[w] + hh) >> sh) & 0x00FF00FFu) << 8);
+      uint8_t* q = out + t * nchan + (i - t * per) * (4 * W);
+      if constexpr (W == 4) *reinterpret_cast<uint4*>(q) = make_uint4(o[0], o[1], o[2], o[3]);
+      else *reinterpret_cast<uint32_t*>(q) = o[0];
     }
-  } else if (layout == TX_LAYOUT_TF) {
-    const int64_t total = nout * nchan;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-      const int64_t t = i / nchan;
-      const int c = (int)(i - t * nchan);
-      uint32_t sum = 0;
-      for (int k = 0; k < f; ++k) sum += in[(t * f + k) * nchan + c];
-      out[t * nchan + c] = (uint8_t)((sum + half) / f);
+  } else if constexpr (MODE == 1) {
+    // rows are a multiple of four samples: the block is one run of words
+    const uint32_t* w = reinterpret_cast<const uint32_t*>(in);
+    if (f == 2) {
+      for (int64_t i = first; i < nchan * n / 4; i += stride) {
+        const uint32_t v = __ldg(w + i);
+        const uint32_t s = (((v & 0x00FF00FFu) + ((v >> 8) & 0x00FF00FFu) + 0x10001u) >> 1) & 0x00FF00FFu;
+        reinterpret_cast<uint16_t*>(out)[i] = (uint16_t)(s | (s >> 8));
+      }
+    } else {
+      const int wf = f >> 2;
+      for (int64_t i = first; i < nchan * nout; i += stride) {
+        uint32_t s = half;
+#pragma unroll 4
+        for (int k = 0; k < wf; ++k) s = __dp4a(__ldg(w + i * wf + k), 0x01010101u, s);
+        out[i] = (uint8_t)(s >> sh);
+      }
     }
   } else {
-    const int64_t total = nout * nchan;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < total; i += stride) {
-      const int c = (int)(i / nout);
-      const int64_t t = i - (int64_t)c * nout;
-      const uint8_t* src = in + (int64_t)c * n + t * f;
-      uint32_t sum = 0;
-      for (int k = 0; k < f; ++k) sum += src[k];
-      out[(int64_t)c * nout + t] = (uint8_t)((sum + half) / f);
+    for (int64_t i = first; i < nout * nchan; i += stride) {
+      uint32_t sum = half;
+      if (layout == TX_LAYOUT_TF) {
+        const int64_t t = i / nchan;
+        const uint8_t* src = in + (t << sh) * nchan + (i - t * nchan);
+        for (int k = 0; k < f; ++k) sum += src[(int64_t)k * nchan];
+      } else {
+        const uint8_t* src = in + (i << sh);   // rows of a whole number of outputs
+        for (int k = 0; k < f; ++k) sum += src[k];
+      }
+      out[i] = (uint8_t)(sum >> sh);
     }
   }
+}
+
+inline int downsample_mode(const void* in, const void* out, int layout, int nchan, int64_t n, int sh) {
+  const uintptr_t a = (uintptr_t)in | (uintptr_t)out;
+  if (layout == TX_LAYOUT_TF) return sh > 8 ? 0 : nchan % 16 == 0 && a % 16 == 0 ? 3 : nchan % 4 == 0 && a % 4 == 0 ? 2 : 0;
+  return sh >= 1 && n % 4 == 0 && a % 4 == 0 ? 1 : 0;
 }
 
 // ---------------------------------------------------------------------------
