@@ -658,12 +658,15 @@ k_stage1(const Src src, const int32_t* __restrict__ uoff, const int32_t* __restr
       for (int c = warp; c < a.m; c += kStage1Warps) {
         int64_t p = a.start + it.tau0 + wrow[w * TSL + c];
         while (p >= R) p -= R;
-        const int pa = (int)p & ~15;
         const uint8_t* row = a.ring + (size_t)(it.s * a.m + c) * R;
         uint8_t* dst = raw + (size_t)c * RB;
-        const int first = min(RB, R - pa);
-        bulk_g2s(dst, row + pa, (uint32_t)first, &barr);
-        if (first < RB) bulk_g2s(dst + first, row, (uint32_t)(RB - first), &barr);
+        int from = (int)p & ~15;
+        for (int done = 0; done < RB;) {   // in pieces where the window wraps (a short ring more than once)
+          const int len = min(RB - done, R - from);
+          bulk_g2s(dst + done, row + from, (uint32_t)len, &barr);
+          done += len;
+          from = 0;
+        }
       }
     }
   };
