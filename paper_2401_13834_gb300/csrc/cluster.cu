@@ -589,7 +589,13 @@ int32_t tx_clusterer_create(const tx_plan* p, double radius_ms, int32_t k, int64
     }
     if (most <= kMaxRows && (int64_t)p->ndm * (most + 1) <= kMaxReach && radius_ms / C->tsamp_ms < 5e8) {
       C->nrow = most;
-      reach.assign((size_t)p->ndm * (most + 1), -1);
+      try {
+        reach.assign((size_t)p->ndm * (most + 1), -1);
+      } catch (const std::bad_alloc&) {
+        set_error("out of host memory");
+        tx_clusterer_destroy(C);
+        return TX_ERR_OOM;
+      }
       for (int d = 0; d < p->ndm; ++d)
         for (int i = 0; i <= most && d + i < p->ndm; ++i) {
           const double gx = x[d + i] - x[d];
