@@ -380,6 +380,7 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
   // (a shorter tile asked for is taken as asked)
   p->s1w = wide1_shape(m, 8);
   p->wide1 = q1 < 256 && stage1_smem_bytes(m, 2 * q1) > kSmemMax && p->s1w.nst >= 2;
+  const bool integer = p->interm != TX_INTERM_F32;   // the float path has its own list
   do {
     p->items1.clear();
     p->tab1.clear();
@@ -390,7 +391,7 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
     // of 64 plus a multiple of T, and R a multiple of 64
     p->tab1_phase = (int32_t)((16 - p->L % 16) % 16);
     const int TS1 = (m + 3) & ~3, SW1 = kStage1StagedWords(q1);
-    for (int s = 0; s < nsub; ++s) {
+    for (int s = 0; s < nsub && integer; ++s) {
       int kb = 0;
       while (kb < nk) {
         auto spread = [&](int k0, int k1) {  // max_c d1[k1-1][c] - d1[k0][c]
@@ -427,7 +428,7 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
     }
     // few items: shorter tiles of the wide kernel keep the SMs busy
     const Wide1Shape next = wide1_shape(m, p->s1w.vw / 2);
-    if (!p->wide1 || p->items1.size() >= (size_t)kWide1MinItems || p->s1w.vw <= 2 || next.nst < 2) break;
+    if (!integer || !p->wide1 || p->items1.size() >= (size_t)kWide1MinItems || p->s1w.vw <= 2 || next.nst < 2) break;
     p->s1w = next;
   } while (true);
   // Time-major order: blocks working at the same time read overlapping input
