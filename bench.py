@@ -183,6 +183,7 @@ class ClockSampler:
 KERNEL_SECTIONS = {
     "k_ingest_tf": "// ingest (",
     "k_stage1": "// stage 1 (",
+    "k_stage1_wide": "// stage 1 of wide sub-bands",
     "k_stage2_u16": "// stage 2 (",
     "k_stage2_pipe": "// stage 2 (",
     "k_boxcar": "// boxcar matched filter",
@@ -206,6 +207,12 @@ def kernel_sha(kernel):
     with open(os.path.join(csrc, "tx_internal.h")) as fh:
         h.update("\n".join(ln for ln in fh.read().split("\n") if ln.startswith("constexpr")).encode())
     return h.hexdigest()[:16]
+
+
+def stage1_kernel(plan):
+    """The integer stage 1 that a plan with the default tile runs (plan.cpp's rule)."""
+    m = plan.nchan // plan.nsub
+    return "k_stage1_wide" if m > 64 or (m > 32 and plan.nsamp % 16 == 0) else "k_stage1"
 
 
 def profiled_traffic(kernel, workload):
@@ -713,7 +720,7 @@ def run_ours(args):
             kernel_of = {"ingest": "k_norm_ingest_tf", "stage1": "k_stage1_f32", "stage2": "k_stage2_pipe32",
                          "stats": "k_stats_f32", "boxcar": "k_boxcar_f32"}
         else:
-            kernel_of = {"ingest": "k_ingest_tf", "stage1": "k_stage1", "stage2": "k_stage2_pipe" if plan.tile_split2
+            kernel_of = {"ingest": "k_ingest_tf", "stage1": stage1_kernel(plan), "stage2": "k_stage2_pipe" if plan.tile_split2
                          and plan.group <= 16 and plan.interm in ("u16", "f16") else
                          ("k_stage2_u16" if plan.interm in ("u16", "f16") else "k_stage2_pipe32"),
                          "stats": "k_stats", "boxcar": "k_boxcar"}
@@ -1010,7 +1017,7 @@ def run_batched(args):
         dom = max(phase_ms, key=phase_ms.get)
         d = phases[dom]
         roof = {"bound": d["bound"], "achieved": d.get("achieved"), "peak": d.get("peak"), "unit": d.get("unit"),
-                "frac": d.get("frac"), "traffic": None, "kernel": {"stage1": "k_stage1", "stage2": "k_stage2_pipe / k_stage2_u16",
+                "frac": d.get("frac"), "traffic": None, "kernel": {"stage1": "k_stage1_wide / k_stage1", "stage2": "k_stage2_pipe / k_stage2_u16",
                                                                       "boxcar": "k_boxcar", "ingest": "k_ingest_batch",
                                                                       "stats": "k_stats"}[dom],
                 "peak_source": (f"{peak_kind} HBM copy bandwidth (MEASURED_PEAKS.json)" if d["bound"] == "hbm" else

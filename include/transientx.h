@@ -131,7 +131,9 @@ typedef struct tx_plan_desc {
   /* Tile shapes (results do not depend on them; 0 = automatic choice):     */
   int32_t        tile_q1;        /* stage-1 tile of 4 * tile_q1 samples: 32, 64, 128
                                     or 256 (must fit shared memory); 0 = the
-                                    largest that fits                               */
+                                    largest that fits. Sub-bands whose largest is
+                                    shorter than 256 run a kernel that sizes itself,
+                                    unless a smaller tile than that is asked for    */
   int32_t        tile_split2;    /* stage-2 warps per fine DM: 1 (tiles of 512
                                     outputs) or 2, 4, 8 (tiles of 1024), with
                                     min(group, 32) * tile_split2 <= 32; 0 = 8, 4, 2
@@ -492,8 +494,9 @@ void tx_batch_destroy(tx_batch* batch);
    is the canonical index of its first core point; a non-core point next to
    several clusters joins the one of smallest id. Results do not depend on the
    order of the input records. The paper searches neighbours with a kd-tree;
-   here a uniform grid of cells of side ~radius_ms does it (section 2.5's
-   prune rules become "only the 3 x 3 cells around a point"). */
+   here each DM trial's points are a row sorted by time, of which a point's
+   neighbours are one interval per row within radius_ms of its DM (a uniform
+   grid of cells of side ~radius_ms where more than 256 trials lie that near). */
 typedef struct tx_cluster {
   int32_t id;                 /* canonical index of the cluster's first core point     */
   int32_t dm_index, t, w_index;

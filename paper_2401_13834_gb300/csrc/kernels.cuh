@@ -10,6 +10,7 @@
 //                tail (time-major input is transposed on the way); nothing is
 //                shifted, the buffer start advances by T instead.
 //   k_stage1     stage 1: P[k][s][t] = sum_{c in s} X[c][t + d1[k][c]]
+//                (k_stage1_wide for sub-bands of many channels)
 //   k_stage2_*   stage 2: D[d][t] = sum_s P[k(d)][s][t + d2[d][s]], plus exact
 //                per-tile sums of D and D^2
 //   k_stats      mean / sigma per DM (block or running) and the per-width
@@ -953,8 +954,10 @@ struct Wide1Shared {
 // `nst` shared-memory stages without block-wide barriers:
 //   * kWide1Producers warps bulk-copy (TMA) the channels' input windows, one
 //     byte per sample from 16-byte aligned ring positions (in pieces where a
-//     window wraps the ring's end), and write per coarse DM the channels' word
-//     offsets, sorted by the residue mod 4 of their byte offsets;
+//     window wraps the ring's end), and per coarse DM the channels' word
+//     offsets, sorted by the residue mod 4 of their byte offsets: the plan's
+//     rows while the window starts keep the phase they were built for, else
+//     sorted here;
 //   * each consumer warp sums whole coarse DMs: kk = its number less a rotating
 //     base, + kWide1Consumers ..., so that work evens out over items.
 // An output word j of lane l holds the four sums of samples 4 (l + 32 j) .. + 3.
@@ -966,16 +969,15 @@ struct Wide1Shared {
 //   sum w = sum(even bytes) + 256 * sum(odd bytes)   (mod 2^32)
 // with the odd bytes accumulated separately as 16-bit lanes, exact for up to
 // 257 channels. Consecutive outputs leave as one 8-byte store.
-// Used for sub-bands of more than 64 channels: k_stage1 rearranges an item's
-// windows into 32-bit words four times their size, which leaves such
-// sub-bands tiles of 512 or 256 outputs and few coarse DMs to share them; one
-// byte per sample lets them keep 512 outputs, 64 coarse DMs and a second item
-// in flight. 125 channels per sub-band (1000 channels, 76 coarse DMs, 20160
-// samples): 231 -> 102 us; 96 channels (937 DMs in groups of 2, 17408 samples):
-// 128 -> 103 us. Both are bound by shared memory (a byte per sample-add) and issue; at 64
-// channels k_stage1's longest tile fits and its rearranged words need fewer
-// instructions: 2.70 against 2.73 ms on the MeerKAT-L block, 14.5 against 16.2
-// us on 16 channels per sub-band.
+// Bound by shared memory (a byte per sample-add: 1.76 ms on the MeerKAT-L block
+// of 64 channels per sub-band) and issue together. k_stage1 rearranges an item's
+// windows into 32-bit words four times their size; here they stay bytes, which
+// leaves room for a second item in flight and, past 64 channels, for tiles of
+// 512 outputs and 64 coarse DMs where k_stage1's shrink. Measured, k_stage1 and
+// this: MeerKAT-L block 2.70 and 2.49 ms (2.73 with the rows sorted here);
+// 1024 channels of 64 per sub-band, 1024 DMs, 32768 samples 403 and 351 us;
+// 125 channels per sub-band (1000 channels, 76 coarse DMs, 20160 samples) 231
+// and 98 us; 96 channels (937 DMs in groups of 2, 17408 samples) 128 and 103 us.
 // Waits are bounded as in k_stage2_pipe; only one producer warp waits for free
 // stages, the others follow it through a named barrier.
 template <int VW, typename PT, typename Src, bool HALF = false>
@@ -1033,8 +1035,10 @@ k_stage1_wide(const Src src, const int32_t* __restrict__ uoff, const int32_t* __
               sh.beam[st] = cur.beam;
             }
             const BeamArgs a = src.get(cur.beam);
-            sh.desc[st] = a.items[lu];
-            mbar_expect_only(&sh.full[st], (uint32_t)(a.m * sp.rb));
+            const Stage1Item it = a.items[lu];
+            sh.desc[st] = it;
+            const bool pre = a.tab1 != nullptr && (int)(a.start & 15) == a.tab1_phase;
+            mbar_expect_only(&sh.full[st], (uint32_t)(a.m * sp.rb + (pre ? (it.ke - it.kb) * sp.tsu * 4 : 0)));
             nextv = (int)gridDim.x + atomicAdd(ictr, 1);
           }
         }
@@ -1068,9 +1072,15 @@ k_stage1_wide(const Src src, const int32_t* __restrict__ uoff, const int32_t* __
         }
       }
       uint32_t* tab = reinterpret_cast<uint32_t*>(raw + (size_t)m * sp.rb);
-      const int lead = (int)((a.start + it.tau0) & 15);
-      if (m <= 128) wide1_rows<4, 2>(d1b, a.nchan, m, n, lead, sp.rb, sp.tsu, tab, pw, lane);
-      else wide1_rows<9, 1>(d1b, a.nchan, m, n, lead, sp.rb, sp.tsu, tab, pw, lane);
+      const int lead = (int)(a.start & 15);   // (tau0 is a multiple of 16)
+      if (a.tab1 != nullptr && lead == a.tab1_phase) {   // the plan's rows
+        if (ptid == kWide1Producers * 32 - 1)
+          bulk_g2s(tab, a.tab1 + it.tab, (uint32_t)(n * sp.tsu) * 4u, &sh.full[st]);
+      } else if (m <= 128) {
+        wide1_rows<4, 2>(d1b, a.nchan, m, n, lead, sp.rb, sp.tsu, tab, pw, lane);
+      } else {
+        wide1_rows<9, 1>(d1b, a.nchan, m, n, lead, sp.rb, sp.tsu, tab, pw, lane);
+      }
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh.full[st]);
       ++q;

@@ -28,8 +28,7 @@ constexpr int kStage1Warps = 32;
 // bytes rounded up to 16-byte chunks.
 constexpr int kStage1StagedWords(int q) { return 2 * q + 4; }
 constexpr int kStage1RawBytes(int q) { return (5 * q + 2 + 15) / 16 * 16; }
-// Sub-bands of more than 64 channels (those whose longest tile above is shorter
-// than 1024 samples): a coarse DM's tile is `vw` 32-bit words per lane of a
+// k_stage1_wide: a coarse DM's tile is `vw` 32-bit words per lane of a
 // warp, four consecutive samples to a word. The last 16 of a tile's samples are
 // slack (see k_stage1_wide) and belong to the next tile.
 constexpr int kWide1Consumers = 28;    // consumer warps
@@ -131,7 +130,7 @@ struct DevicePlan {
 
 void set_error(const char* fmt, ...);
 int64_t stage1_smem_bytes(int m, int q);
-// The wide sub-bands' stage 1 for m channels, at most `most` words per lane: words per lane, the delay spread
+// k_stage1_wide's shape for m channels and at most `most` words per lane: words per lane, the delay spread
 // and coarse DMs an item may have, bytes of a channel's window, words of a
 // coarse DM's offset row, bytes of a stage and how many fit.
 struct Wide1Shape {
@@ -211,7 +210,8 @@ struct tx_plan {
   // words, word c = c * staged words + ((tab1_phase + d1[kb][c]) & 15) +
   // d1[kb + kk][c] - d1[kb][c], then abase[kb + kk][s] for kk < ke - kb
   // (padded to 4); valid for executes whose window start has tab1_phase as
-  // its residue mod 16 (every block when T is a multiple of 16)
+  // its residue mod 16 (every block when T is a multiple of 16). The wide
+  // kernel's are s1w.tsu words a row as wide1_rows writes them, without abase
   std::vector<int32_t> tab1;
   int32_t tab1_phase = 0;
   // pipelined stage 2 (16 and 32 bits), per (coarse group k, sub-band chunk): rows g < group of

@@ -1,4 +1,4 @@
-"""Stage 1 of sub-bands of more than 64 channels at the sizes where it can go
+"""Stage 1 of sub-bands of many channels (k_stage1_wide) at the sizes where it can go
 wrong: each length of its tiles, residues and spreads of every kind, coarse DMs
 that fill an item and one more, blocks of one sample, rings shorter than a
 window, lengths that give the windows every phase, every form of the
@@ -35,10 +35,14 @@ def _want(X, op, plan, b):
 SHAPES = [(65, 2, 20, 60.0, 1, False), (70, 1, 140, 40.0, 2500, True), (96, 2, 70, 900.0, 1000, False),
           (125, 2, 66, 90.0, 1531, True), (128, 1, 130, 200.0, 777, False), (160, 1, 36, 60.0, 1111, False),
           (200, 1, 70, 300.0, 640, True), (257, 2, 40, 120.0, 333, False)]
+# lengths of whole 16 samples: the plan's offset rows, from 33 channels on (64 * 2 coarse DMs: two full items)
+ROWS = [(33, 2, 20, 60.0, 16, False), (33, 1, 256, 40.0, 2512, True), (40, 2, 70, 900.0, 1008, False),
+        (64, 2, 66, 90.0, 1536, True), (64, 1, 130, 200.0, 784, False), (64, 2, 40, 120.0, 779, False),
+        (125, 2, 66, 90.0, 1536, False), (160, 1, 36, 60.0, 1120, True), (257, 1, 40, 120.0, 336, False)]
 
 
 @pytest.mark.parametrize("interm", ["u16", "i32"])
-@pytest.mark.parametrize("shape", SHAPES)
+@pytest.mark.parametrize("shape", SHAPES + ROWS)
 def test_series_equal_the_oracle(tx, shape, interm):  # noqa: F811
     wl, plan, op, X = _setup(tx, *shape[:5], interm, shape[5])
     L, T = plan.overlap, plan.nsamp
@@ -51,8 +55,9 @@ def test_series_equal_the_oracle(tx, shape, interm):  # noqa: F811
     assert beam.failed() == 0
 
 
-def test_noalloc_equals_the_oracle(tx):  # noqa: F811
-    wl, plan, op, X = _setup(tx, 100, 2, 20, 60.0, 900, "u16")
+@pytest.mark.parametrize("m,nsamp", [(100, 900), (100, 912), (64, 912)])
+def test_noalloc_equals_the_oracle(tx, m, nsamp):  # noqa: F811
+    wl, plan, op, X = _setup(tx, m, 2, 20, 60.0, nsamp, "u16")
     n = plan.overlap + plan.nsamp
     ld = (n + 63) // 64 * 64
     x = torch.zeros((wl.nchan, ld), dtype=torch.uint8, device="cuda")
@@ -63,10 +68,11 @@ def test_noalloc_equals_the_oracle(tx):  # noqa: F811
 
 
 def test_batch_of_unlike_beams(tx):  # noqa: F811
-    """Wide beams of several shapes and forms, compact and full, beside a narrow one."""
+    """Beams of several shapes and forms, compact and full, beside narrow ones; rows of the plan and sorted rows."""
     made = [_setup(tx, *s) for s in [(96, 2, 30, 60.0, 900, "u16"), (125, 1, 40, 80.0, 1100, "u16"),
                                      (96, 1, 50, 30.0, 513, "f16"), (16, 4, 24, 60.0, 800, "u16"),
-                                     (125, 2, 20, 50.0, 640, "f16")]]
+                                     (125, 2, 20, 50.0, 640, "f16"), (64, 2, 24, 60.0, 640, "u16"),
+                                     (64, 2, 24, 60.0, 650, "u16"), (40, 2, 30, 70.0, 656, "f16")]]
     plans = [p for _, p, _, _ in made]
     beams = [tx.Beam(p, compact=i % 2 == 0) for i, p in enumerate(plans)]
     for (_, p, _, X), bm in zip(made, beams):
