@@ -212,7 +212,7 @@ def kernel_sha(kernel):
 def stage1_kernel(plan):
     """The integer stage 1 that a plan with the default tile runs (plan.cpp's rule)."""
     m = plan.nchan // plan.nsub
-    return "k_stage1_wide" if m > 64 or (m > 32 and plan.nsamp % 16 == 0) else "k_stage1"
+    return "k_stage1_wide" if m >= 16 else "k_stage1"
 
 
 def profiled_traffic(kernel, workload):

@@ -131,9 +131,9 @@ typedef struct tx_plan_desc {
   /* Tile shapes (results do not depend on them; 0 = automatic choice):     */
   int32_t        tile_q1;        /* stage-1 tile of 4 * tile_q1 samples: 32, 64, 128
                                     or 256 (must fit shared memory); 0 = the
-                                    largest that fits. Sub-bands whose largest is
-                                    shorter than 256 run a kernel that sizes itself,
-                                    unless a smaller tile than that is asked for    */
+                                    largest that fits. At that largest one sub-bands of
+                                    16 channels and more run a kernel that sizes
+                                    itself                                          */
   int32_t        tile_split2;    /* stage-2 warps per fine DM: 1 (tiles of 512
                                     outputs) or 2, 4, 8 (tiles of 1024), with
                                     min(group, 32) * tile_split2 <= 32; 0 = 8, 4, 2

@@ -139,24 +139,20 @@ void launch_stage1_t(const tx_plan* p, const BeamArgs& a, int32_t* ictr, cudaStr
 }
 
 template <int VW, typename PT, bool HALF = false>
-void launch_wide1_t(const tx_plan* p, const BeamArgs& a, int32_t* ictr, cudaStream_t st, bool pdl) {
+void launch_wide1_t(const tx_plan* p, const BeamArgs& a, int32_t* ictr, cudaStream_t st) {
   const int nitems = (int)p->items1.size();
   const int grid = std::min(nitems, std::max(p->dev.num_sms, 1));
-  if (pdl)
-    launch_pdl(k_stage1_wide<VW, PT, OneBeam, HALF>, grid, kWide1Warps * 32, (size_t)p->s1w.smem(), st, OneBeam{a},
-               nullptr, nullptr, 1, nitems, p->s1w, 1u, ictr);
-  else
-    k_stage1_wide<VW, PT, OneBeam, HALF><<<grid, kWide1Warps * 32, p->s1w.smem(), st>>>(
-        OneBeam{a}, nullptr, nullptr, 1, nitems, p->s1w, 1u, ictr);
+  launch_pdl(k_stage1_wide<VW, PT, OneBeam, HALF>, grid, kWide1Warps * 32, (size_t)p->s1w.smem(), st, OneBeam{a},
+             nullptr, nullptr, 1, nitems, p->s1w, 1u, ictr);
 }
 
 // stage 1 of a plan of wide sub-bands with its item counter
 template <typename PT, bool HALF = false>
-void launch_wide1(const tx_plan* p, const BeamArgs& a, int32_t* ictr, cudaStream_t st, bool pdl = true) {
+void launch_wide1(const tx_plan* p, const BeamArgs& a, int32_t* ictr, cudaStream_t st) {
   switch (p->s1w.vw) {
-    case 8: launch_wide1_t<8, PT, HALF>(p, a, ictr, st, pdl); break;
-    case 4: launch_wide1_t<4, PT, HALF>(p, a, ictr, st, pdl); break;
-    default: launch_wide1_t<2, PT, HALF>(p, a, ictr, st, pdl); break;
+    case 8: launch_wide1_t<8, PT, HALF>(p, a, ictr, st); break;
+    case 4: launch_wide1_t<4, PT, HALF>(p, a, ictr, st); break;
+    default: launch_wide1_t<2, PT, HALF>(p, a, ictr, st); break;
   }
 }
 
@@ -828,7 +824,7 @@ int32_t tx_dedisperse_noalloc(const tx_plan* p, const uint8_t* d_x, int64_t ld, 
     return TX_ERR_INVALID_ARG;
   }
   // scratch layout: stage-1 work items, d1, abase, e2, stage-1 sums, per-tile sums
-  const size_t b_items = align256(p->items1.size() * sizeof(Stage1Item));
+  const size_t b_items = align256(p->items_na.size() * sizeof(Stage1Item));
   const size_t b_d1 = align256(p->d1.size() * 4);
   const size_t b_abase = align256(p->abase.size() * 4);
   const size_t b_e2 = align256(p->e2.size() * 4);
@@ -858,7 +854,7 @@ int32_t tx_dedisperse_noalloc(const tx_plan* p, const uint8_t* d_x, int64_t ld, 
   int32_t* tab2 = reinterpret_cast<int32_t*>(base + b_items + b_d1 + b_abase + b_e2 + b_P + b_part);
   int32_t* ictr = reinterpret_cast<int32_t*>(base + b_items + b_d1 + b_abase + b_e2 + b_P + b_part + b_tab2);
   cudaStream_t st = (cudaStream_t)stream;
-  TX_CUDA(cudaMemcpyAsync(items, p->items1.data(), p->items1.size() * sizeof(Stage1Item), cudaMemcpyHostToDevice, st));
+  TX_CUDA(cudaMemcpyAsync(items, p->items_na.data(), p->items_na.size() * sizeof(Stage1Item), cudaMemcpyHostToDevice, st));
   TX_CUDA(cudaMemcpyAsync(d1, p->d1.data(), p->d1.size() * 4, cudaMemcpyHostToDevice, st));
   TX_CUDA(cudaMemcpyAsync(abase, p->abase.data(), p->abase.size() * 4, cudaMemcpyHostToDevice, st));
   TX_CUDA(cudaMemcpyAsync(e2, p->e2.data(), p->e2.size() * 4, cudaMemcpyHostToDevice, st));
@@ -896,7 +892,7 @@ int32_t tx_dedisperse_noalloc(const tx_plan* p, const uint8_t* d_x, int64_t ld, 
   a.polls = first_wait_polls();   // a wait that gives up counts in tx_wait_timeouts only
 
   // stage 1
-  const int nitems = (int)p->items1.size();
+  const int nitems = (int)p->items_na.size();
   const int smem1 = (int)stage1_smem_bytes(p->m, p->q1);
   const int grid1 = std::min(nitems, std::max(nsm, 1));
   TX_CUDA(cudaMemsetAsync(ictr, 0, sizeof(int32_t), st));
@@ -906,9 +902,7 @@ int32_t tx_dedisperse_noalloc(const tx_plan* p, const uint8_t* d_x, int64_t ld, 
     k_stage1<Q, uint16_t, OneBeam><<<grid1, kStage1Warps * 32, smem1, st>>>(OneBeam{a}, nullptr, nullptr, 1, nitems, \
                                                                             p->m, 1u, ictr);                  \
   } while (0)
-  if (p->wide1) {
-    launch_wide1<uint16_t>(p, a, ictr, st, false);
-  } else switch (p->q1) {
+  switch (p->q1) {
     case 256: TX_NA_S1(256); break;
     case 128: TX_NA_S1(128); break;
     case 64: TX_NA_S1(64); break;

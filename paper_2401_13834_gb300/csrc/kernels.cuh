@@ -880,64 +880,13 @@ __device__ __forceinline__ void wide1_shift(uint32_t (&aw)[VW], uint32_t (&ah)[V
   }
 }
 
-// Offset rows of the coarse DMs kk = pw, pw + kWide1Producers ... of an item:
-// {residue 3 | residue 2 << 16, residue 1 | residue 0 << 16} counts, then the
-// channels' byte offsets (of words) residue by residue, each part padded to four
-// entries. NCH: groups of 32 channels (m <= 32 NCH); KB coarse DMs' delays are
-// loaded at once. lead: the window start's residue mod 16; rb: bytes per channel.
-template <int NCH, int KB>
-__device__ __forceinline__ void wide1_rows(const int32_t* __restrict__ d1b, int nchan, int m, int n, int lead, int rb,
-                                            int tsu, uint32_t* __restrict__ tab, int pw, int lane) {
-  int d0[NCH];
-#pragma unroll
-  for (int g = 0; g < NCH; ++g) d0[g] = 32 * g + lane < m ? __ldg(d1b + 32 * g + lane) : 0;
-  const unsigned below = (1u << lane) - 1u;
-  for (int k0 = pw; k0 < n; k0 += kWide1Producers * KB) {
-    int x[KB][NCH];   // byte offsets of the channels' first samples; -1: no channel
-#pragma unroll
-    for (int i = 0; i < KB; ++i) {
-      const int32_t* d1k = d1b + (size_t)min(k0 + i * kWide1Producers, n - 1) * nchan;
-#pragma unroll
-      for (int g = 0; g < NCH; ++g) x[i][g] = 32 * g + lane < m ? __ldg(d1k + 32 * g + lane) : 0;
-    }
-#pragma unroll
-    for (int i = 0; i < KB; ++i) {
-      const int kk = k0 + i * kWide1Producers;
-      if (kk >= n) break;
-      uint32_t* row = tab + kk * tsu;
-      int cnt[4] = {0, 0, 0, 0};
-#pragma unroll
-      for (int g = 0; g < NCH; ++g) {
-        if (32 * g >= m) break;
-        x[i][g] = 32 * g + lane < m ? ((lead + d0[g]) & 15) + x[i][g] - d0[g] : -1;
-#pragma unroll
-        for (int r = 0; r < 4; ++r)
-          cnt[r] += __popc(__ballot_sync(0xffffffffu, x[i][g] >= 0 && (x[i][g] & 3) == r));
-      }
-      int at[4];
-      at[3] = 4;
-      at[2] = at[3] + ((cnt[3] + 3) & ~3);
-      at[1] = at[2] + ((cnt[2] + 3) & ~3);
-      at[0] = at[1] + ((cnt[1] + 3) & ~3);
-      if (lane == 0)
-        *reinterpret_cast<uint2*>(row) =
-            make_uint2((uint32_t)cnt[3] | (uint32_t)cnt[2] << 16, (uint32_t)cnt[1] | (uint32_t)cnt[0] << 16);
-#pragma unroll
-      for (int g = 0; g < NCH; ++g) {
-        if (32 * g >= m) break;
-        int pos = 0;
-#pragma unroll
-        for (int r = 0; r < 4; ++r) {
-          const bool in = x[i][g] >= 0 && (x[i][g] & 3) == r;
-          const unsigned b = __ballot_sync(0xffffffffu, in);
-          if (in) pos = at[r] + __popc(b & below);
-          at[r] += __popc(b);
-        }
-        if (x[i][g] >= 0) row[pos] = (uint32_t)((32 * g + lane) * rb + (x[i][g] & ~3));
-      }
-    }
-  }
-}
+// Samples by which the tiles of a beam's execute start before their items': the
+// plan's rows hold for window starts of one residue mod 16, so where a block
+// starts at another one (lengths that are no multiples of 16; a caller's buffer)
+// the whole tiling moves to the front instead of the rows being rebuilt (up to
+// three more shifts a tile; sorting rows in the kernel took 98 us instead of 82
+// at 125 channels per sub-band and a length of 20011).
+__device__ __forceinline__ int wide1_early(const BeamArgs& a) { return (int)((a.start - a.tab1_phase) & 15); }
 
 // What the roles of a block hand each other.
 struct Wide1Shared {
@@ -955,9 +904,7 @@ struct Wide1Shared {
 //   * kWide1Producers warps bulk-copy (TMA) the channels' input windows, one
 //     byte per sample from 16-byte aligned ring positions (in pieces where a
 //     window wraps the ring's end), and per coarse DM the channels' word
-//     offsets, sorted by the residue mod 4 of their byte offsets: the plan's
-//     rows while the window starts keep the phase they were built for, else
-//     sorted here;
+//     offsets, sorted by the residue mod 4 of their byte offsets (the plan's);
 //   * each consumer warp sums whole coarse DMs: kk = its number less a rotating
 //     base, + kWide1Consumers ..., so that work evens out over items.
 // An output word j of lane l holds the four sums of samples 4 (l + 32 j) .. + 3.
@@ -974,10 +921,9 @@ struct Wide1Shared {
 // windows into 32-bit words four times their size; here they stay bytes, which
 // leaves room for a second item in flight and, past 64 channels, for tiles of
 // 512 outputs and 64 coarse DMs where k_stage1's shrink. Measured, k_stage1 and
-// this: MeerKAT-L block 2.70 and 2.49 ms (2.73 with the rows sorted here);
-// 1024 channels of 64 per sub-band, 1024 DMs, 32768 samples 403 and 351 us;
-// 125 channels per sub-band (1000 channels, 76 coarse DMs, 20160 samples) 231
-// and 98 us; 96 channels (937 DMs in groups of 2, 17408 samples) 128 and 103 us.
+// this: MeerKAT-L block 2.70 and 2.49 ms; 1024 channels of 64 per sub-band, 1024
+// DMs, 32768 samples 403 and 350 us (32771 samples 419 and 360); 125 channels per
+// sub-band (1000 channels, 76 coarse DMs, 20160 samples) 231 and 82 us.
 // Waits are bounded as in k_stage2_pipe; only one producer warp waits for free
 // stages, the others follow it through a named barrier.
 template <int VW, typename PT, typename Src, bool HALF = false>
@@ -1037,8 +983,7 @@ k_stage1_wide(const Src src, const int32_t* __restrict__ uoff, const int32_t* __
             const BeamArgs a = src.get(cur.beam);
             const Stage1Item it = a.items[lu];
             sh.desc[st] = it;
-            const bool pre = a.tab1 != nullptr && (int)(a.start & 15) == a.tab1_phase;
-            mbar_expect_only(&sh.full[st], (uint32_t)(a.m * sp.rb + (pre ? (it.ke - it.kb) * sp.tsu * 4 : 0)));
+            mbar_expect_only(&sh.full[st], (uint32_t)(a.m * sp.rb + (it.ke - it.kb) * sp.tsu * 4));
             nextv = (int)gridDim.x + atomicAdd(ictr, 1);
           }
         }
@@ -1060,8 +1005,9 @@ k_stage1_wide(const Src src, const int32_t* __restrict__ uoff, const int32_t* __
       fence_proxy_async();
       for (int c = ptid; c < m; c += kWide1Producers * 32) {
         const int R = (int)a.R;
-        int64_t p = a.start + it.tau0 + __ldg(d1b + c);
+        int64_t p = a.start + it.tau0 - wide1_early(a) + __ldg(d1b + c);
         while (p >= R) p -= R;
+        if (p < 0) p += R;   // (feeds samples before the row only)
         const uint8_t* row = a.ring + (size_t)(it.s * m + c) * R;
         int from = (int)p & ~15;
         for (int done = 0; done < sp.rb;) {
@@ -1072,15 +1018,8 @@ k_stage1_wide(const Src src, const int32_t* __restrict__ uoff, const int32_t* __
         }
       }
       uint32_t* tab = reinterpret_cast<uint32_t*>(raw + (size_t)m * sp.rb);
-      const int lead = (int)(a.start & 15);   // (tau0 is a multiple of 16)
-      if (a.tab1 != nullptr && lead == a.tab1_phase) {   // the plan's rows
-        if (ptid == kWide1Producers * 32 - 1)
-          bulk_g2s(tab, a.tab1 + it.tab, (uint32_t)(n * sp.tsu) * 4u, &sh.full[st]);
-      } else if (m <= 128) {
-        wide1_rows<4, 2>(d1b, a.nchan, m, n, lead, sp.rb, sp.tsu, tab, pw, lane);
-      } else {
-        wide1_rows<9, 1>(d1b, a.nchan, m, n, lead, sp.rb, sp.tsu, tab, pw, lane);
-      }
+      if (ptid == kWide1Producers * 32 - 1)
+        bulk_g2s(tab, a.tab1 + it.tab, (uint32_t)(n * sp.tsu) * 4u, &sh.full[st]);
       __syncwarp();
       if (lane == 0) mbar_arrive(&sh.full[st]);
       ++q;
@@ -1111,9 +1050,10 @@ k_stage1_wide(const Src src, const int32_t* __restrict__ uoff, const int32_t* __
     const uint8_t* S = raw + 4 * lane;
     const uint32_t* tab = reinterpret_cast<const uint32_t*>(raw + (size_t)a.m * sp.rb);
     const int off = HALF ? a.hoff[s] : 0;   // the sub-band's offset (half intermediates)
+    const int early = wide1_early(a);
     for (int kk = warp >= base ? warp - base : warp - base + kWide1Consumers; kk < n; kk += kWide1Consumers) {
       const size_t prow = (size_t)(kb + kk) * a.nsub + s;
-      const int rel = tau0 - __ldg(a.abase + prow);   // used after the sums
+      const int rel = tau0 - (early & ~3) - __ldg(a.abase + prow);   // used after the sums
       const uint32_t* row = tab + kk * sp.tsu;
       const uint2 h = *reinterpret_cast<const uint2*>(row);
       const int c3 = (int)(h.x & 0xFFFFu), c2 = (int)(h.x >> 16), c1 = (int)(h.y & 0xFFFFu), c0 = (int)(h.y >> 16);
@@ -1131,7 +1071,8 @@ k_stage1_wide(const Src src, const int32_t* __restrict__ uoff, const int32_t* __
       wide1_shift<VW>(aw, ah, lane);
       e += (c1 + 3) & ~3;
       wide1_add<VW>(aw, ah, S, e, c0, unit);
-      PT* o = static_cast<PT*>(a.P) + prow * a.Pp + (rel + 4 * lane);   // rel and Pp are multiples of 16
+      for (int i = early & 3; i > 0; --i) wide1_shift<VW>(aw, ah, lane);
+      PT* o = static_cast<PT*>(a.P) + prow * a.Pp + (rel + 4 * lane);   // rel is a multiple of 4, Pp of 16
 #pragma unroll
       for (int v = 0; v < VW; ++v) {
         const uint32_t lo = aw[v] - (ah[v] << 8);

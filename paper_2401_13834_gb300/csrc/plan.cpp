@@ -68,9 +68,11 @@ Wide1Shape wide1_shape(int m, int most) {
 }
 
 // Appends the offset rows of the wide stage 1 for sub-band s, coarse DMs [kb, ke)
-// to tab1 (the layout that wide1_rows writes), for windows that start with
-// tab1_phase. The producers' own sorting took the kernel from 2.49 to 2.73 ms on
-// the MeerKAT-L block (64 channels); the rows are 5 MB there.
+// to tab1, for windows that start with tab1_phase: s1w.tsu words each, {channels
+// of residue 3 | residue 2 << 16, residue 1 | residue 0 << 16}, two unused, then
+// the channels' byte offsets (of words) residue by residue, each part but the
+// last padded to four. Rows sorted by the producer warps instead took the kernel
+// from 2.49 to 2.73 ms on the MeerKAT-L block; there the rows are 5 MB.
 static void wide1_table(tx_plan* p, int s, int kb, int ke) {
   const int m = p->m, tsu = p->s1w.tsu;
   const int32_t* d0 = p->d1.data() + (size_t)kb * p->nchan + (size_t)s * m;
@@ -164,6 +166,62 @@ static int32_t float_chunks(tx_plan* p, int s, int kb, int ke) {
     }
   }
   return nchunk;
+}
+
+// The work items of the integer stage 1: the wide kernel's in its shape s1w or
+// k_stage1's, with their offset tables in tab1 where `tab` is set.
+static void stage1_items(tx_plan* p, bool wide, bool tab, std::vector<Stage1Item>& items) {
+  const int m = p->m, nk = p->nk, nsub = p->nsub, nchan = p->nchan, q1 = p->q1;
+  const int span_max = wide ? p->s1w.span : q1 - 16, most = wide ? p->s1w.nmax : kStage1MaxCoarse;
+  const int64_t step = wide ? kWide1TileStep(p->s1w.vw) : 4 * (int64_t)q1;
+  const int TS1 = (m + 3) & ~3, SW1 = kStage1StagedWords(q1);
+  items.clear();
+  if (tab) p->tab1.clear();
+  for (int s = 0; s < nsub; ++s) {
+    int kb = 0;
+    while (kb < nk) {
+      auto spread = [&](int k0, int k1) {  // max_c d1[k1-1][c] - d1[k0][c]
+        int32_t v = 0;
+        for (int c = s * m; c < (s + 1) * m; ++c)
+          v = std::max(v, p->d1[(size_t)(k1 - 1) * nchan + c] - p->d1[(size_t)k0 * nchan + c]);
+        return v;
+      };
+      int ke = kb + 1;
+      while (ke < nk && ke - kb < most && spread(kb, ke + 1) <= span_max) ++ke;
+      // 16, 32 or 64 coarse DMs keep the 32 warps evenly busy (two, one or half a warp per DM)
+      // (the wide kernel evens its warps out over items)
+      if (!wide && ke - kb >= 32) ke = kb + (ke - kb) / 32 * 32;
+      else if (!wide && ke - kb >= 16) ke = kb + 16;
+      const int32_t span = spread(kb, ke);
+      int64_t lo = INT64_MAX, hi = 0;
+      for (int k = kb; k < ke; ++k) {
+        lo = std::min<int64_t>(lo, p->abase[(size_t)k * nsub + s]);
+        hi = std::max<int64_t>(hi, (int64_t)p->abase[(size_t)k * nsub + s] + p->Pp);
+      }
+      if (wide) hi += 12;   // (a multiple of 4 below 16: see wide1_early)
+      const int32_t toff = tab ? (int32_t)p->tab1.size() : 0;
+      if (tab && wide) {
+        wide1_table(p, s, kb, ke);
+      } else if (tab) {
+        for (int kk = 0; kk < ke - kb; ++kk)
+          for (int c = 0; c < TS1; ++c) {
+            if (c >= m) { p->tab1.push_back(0); continue; }
+            const int32_t d0 = p->d1[(size_t)kb * nchan + s * m + c];
+            p->tab1.push_back(c * SW1 + ((p->tab1_phase + d0) & 15) + p->d1[(size_t)(kb + kk) * nchan + s * m + c] - d0);
+          }
+        for (int kk = 0; kk < ((ke - kb + 3) & ~3); ++kk)   // the coarse DMs' P-row bases
+          p->tab1.push_back(kk < ke - kb ? p->abase[(size_t)(kb + kk) * nsub + s] : 0);
+      }
+      for (int64_t t0 = floor_div(lo, step) * step; t0 < hi; t0 += step)
+        items.push_back(Stage1Item{s, kb, ke, (int32_t)t0, span, toff, 0, 0});
+      kb = ke;
+    }
+  }
+  // Time-major order: blocks working at the same time read overlapping input
+  // windows of every sub-band, which keeps the ring's working set in L2.
+  std::stable_sort(items.begin(), items.end(), [](const Stage1Item& a, const Stage1Item& b) {
+    return a.tau0 != b.tau0 ? a.tau0 < b.tau0 : (a.s != b.s ? a.s < b.s : a.kb < b.kb);
+  });
 }
 
 static int build(tx_plan* p, const tx_plan_desc* d) {
@@ -404,69 +462,28 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
   if (stage1_smem_bytes(m, q1) > kSmemMax) { set_error("too many channels per sub-band for stage 1 (%d)", m); return TX_ERR_UNSUPPORTED; }
   p->q1 = q1;
   // The wide kernel, unless a tile shorter than the longest that fits is asked
-  // for: past 64 channels per sub-band (k_stage1's longest tile is then shorter
-  // than 1024 samples: 231 against 98 us at 125 channels) always; from 33 on
-  // where every block keeps the window phase of the plan's rows (64 channels:
-  // 2.49 against 2.70 ms with them, 2.73 without).
+  // for. Stage 1 of k_stage1 and of it: 16 channels per sub-band 1.06 and 0.91 ms
+  // (1024 channels, 4096 DMs, 65536 samples), 32 channels 1.62 and 1.49, 64
+  // channels 2.70 and 2.49 (4096 channels), 125 channels 231 and 82 us (where
+  // k_stage1's tiles shrink to 256 samples). Few channels spread over the four
+  // residues leave little between shifts: below 16 k_stage1 stays.
   p->s1w = wide1_shape(m, 8);
-  p->wide1 = p->s1w.nst >= 2 && (q1 < 256 ? stage1_smem_bytes(m, 2 * q1) > kSmemMax : m > 32 && p->T % 16 == 0);
-  const bool integer = p->interm != TX_INTERM_F32;   // the float path has its own list
-  do {
-    p->items1.clear();
-    p->tab1.clear();
-    p->span1_max = p->wide1 ? p->s1w.span : q1 - 16;
-    const int most1 = p->wide1 ? p->s1w.nmax : kStage1MaxCoarse;
-    const int64_t tt1 = p->wide1 ? kWide1TileStep(p->s1w.vw) : 4 * (int64_t)q1;
-    // every window start of an execute is (head - L) mod R with head a multiple
-    // of 64 plus a multiple of T, and R a multiple of 64
-    p->tab1_phase = (int32_t)((16 - p->L % 16) % 16);
-    const int TS1 = (m + 3) & ~3, SW1 = kStage1StagedWords(q1);
-    for (int s = 0; s < nsub && integer; ++s) {
-      int kb = 0;
-      while (kb < nk) {
-        auto spread = [&](int k0, int k1) {  // max_c d1[k1-1][c] - d1[k0][c]
-          int32_t v = 0;
-          for (int c = s * m; c < (s + 1) * m; ++c)
-            v = std::max(v, p->d1[(size_t)(k1 - 1) * nchan + c] - p->d1[(size_t)k0 * nchan + c]);
-          return v;
-        };
-        int ke = kb + 1;
-        while (ke < nk && ke - kb < most1 && spread(kb, ke + 1) <= p->span1_max) ++ke;
-        // 16, 32 or 64 coarse DMs keep the 32 warps evenly busy (two, one or half a warp per DM)
-        // (the wide kernel evens its warps out over items)
-        if (!p->wide1 && ke - kb >= 32) ke = kb + (ke - kb) / 32 * 32;
-        else if (!p->wide1 && ke - kb >= 16) ke = kb + 16;
-        const int32_t span = spread(kb, ke);
-        int64_t lo = INT64_MAX, hi = 0;
-        for (int k = kb; k < ke; ++k) {
-          lo = std::min<int64_t>(lo, p->abase[(size_t)k * nsub + s]);
-          hi = std::max<int64_t>(hi, (int64_t)p->abase[(size_t)k * nsub + s] + p->Pp);
-        }
-        const int32_t toff = (int32_t)p->tab1.size();
-        for (int kk = 0; kk < ke - kb && !p->wide1; ++kk)
-          for (int c = 0; c < TS1; ++c) {
-            if (c >= m) { p->tab1.push_back(0); continue; }
-            const int32_t d0 = p->d1[(size_t)kb * nchan + s * m + c];
-            p->tab1.push_back(c * SW1 + ((p->tab1_phase + d0) & 15) + p->d1[(size_t)(kb + kk) * nchan + s * m + c] - d0);
-          }
-        if (p->wide1) wide1_table(p, s, kb, ke);
-        for (int kk = 0; kk < ((ke - kb + 3) & ~3) && !p->wide1; ++kk)   // the coarse DMs' P-row bases
-          p->tab1.push_back(kk < ke - kb ? p->abase[(size_t)(kb + kk) * nsub + s] : 0);
-        for (int64_t t0 = floor_div(lo, tt1) * tt1; t0 < hi; t0 += tt1)
-          p->items1.push_back(Stage1Item{s, kb, ke, (int32_t)t0, span, toff, 0, 0});
-        kb = ke;
-      }
-    }
+  p->wide1 = p->s1w.nst >= 2 && (q1 < 256 ? stage1_smem_bytes(m, 2 * q1) > kSmemMax : m >= 16);
+  // every window start of an execute is (head - L) mod R with head a multiple
+  // of 64 plus a multiple of T, and R a multiple of 64
+  p->tab1_phase = (int32_t)((16 - p->L % 16) % 16);
+  while (p->interm != TX_INTERM_F32) {   // (the float path has its own list)
+    stage1_items(p, p->wide1 != 0, true, p->items1);
     // few items: shorter tiles of the wide kernel keep the SMs busy
     const Wide1Shape next = wide1_shape(m, p->s1w.vw / 2);
-    if (!integer || !p->wide1 || p->items1.size() >= (size_t)kWide1MinItems || p->s1w.vw <= 2 || next.nst < 2) break;
+    if (!p->wide1 || p->items1.size() >= (size_t)kWide1MinItems || p->s1w.vw <= 2 || next.nst < 2) break;
     p->s1w = next;
-  } while (true);
-  // Time-major order: blocks working at the same time read overlapping input
-  // windows of every sub-band, which keeps the ring's working set in L2.
-  std::stable_sort(p->items1.begin(), p->items1.end(), [](const Stage1Item& a, const Stage1Item& b) {
-    return a.tau0 != b.tau0 ? a.tau0 < b.tau0 : (a.s != b.s ? a.s < b.s : a.kb < b.kb);
-  });
+  }
+  // tx_dedisperse_noalloc runs k_stage1 in any case: its static scratch has no room for the rows
+  if (p->interm == TX_INTERM_U16) {
+    if (p->wide1) stage1_items(p, false, false, p->items_na);
+    else p->items_na = p->items1;
+  }
   if (p->interm == TX_INTERM_F32) {
     // window starts are (head - L) mod R, head a multiple of 64 plus a multiple of T
     p->phases_f = p->T % 4 == 0 ? 1 : 4;

@@ -32,7 +32,7 @@ constexpr int kStage1RawBytes(int q) { return (5 * q + 2 + 15) / 16 * 16; }
 // warp, four consecutive samples to a word. The last 16 of a tile's samples are
 // slack (see k_stage1_wide) and belong to the next tile.
 constexpr int kWide1Consumers = 28;    // consumer warps
-constexpr int kWide1Producers = 4;     // copying and table-building warps
+constexpr int kWide1Producers = 4;     // copying warps
 constexpr int kWide1Warps = kWide1Consumers + kWide1Producers;
 constexpr int kWide1MaxStages = 8;     // items in flight
 constexpr int kWide1TileStep(int vw) { return 128 * vw - 16; }
@@ -176,7 +176,6 @@ struct tx_plan {
   int64_t R = 0;                  // ring bytes per channel (circular)
   int64_t head0 = 0;              // where a fresh beam's first block lands
   int32_t q1 = 256;               // stage-1 quarter length (words)
-  int32_t span1_max = 256;        // staged delay spread limit of stage 1
   int32_t wide1 = 0;              // stage 1 runs k_stage1_wide in the shape s1w
   tx::Wide1Shape s1w{};
   int32_t span2_max = 0;          // max stage-2 delay spread within a group
@@ -206,12 +205,13 @@ struct tx_plan {
   std::vector<uint32_t> tab_f;
   int32_t phases_f = 1, phase0_f = 0;
   std::vector<tx::Stage1Item> items1;
+  std::vector<tx::Stage1Item> items_na;   // tx_dedisperse_noalloc's, for k_stage1
   // stage-1 offset tables, per (s, kb, ke): rows kk < ke - kb of (m + 3) & ~3
   // words, word c = c * staged words + ((tab1_phase + d1[kb][c]) & 15) +
   // d1[kb + kk][c] - d1[kb][c], then abase[kb + kk][s] for kk < ke - kb
   // (padded to 4); valid for executes whose window start has tab1_phase as
   // its residue mod 16 (every block when T is a multiple of 16). The wide
-  // kernel's are s1w.tsu words a row as wide1_rows writes them, without abase
+  // kernel's: see wide1_table
   std::vector<int32_t> tab1;
   int32_t tab1_phase = 0;
   // pipelined stage 2 (16 and 32 bits), per (coarse group k, sub-band chunk): rows g < group of

@@ -35,8 +35,10 @@ def _want(X, op, plan, b):
 SHAPES = [(65, 2, 20, 60.0, 1, False), (70, 1, 140, 40.0, 2500, True), (96, 2, 70, 900.0, 1000, False),
           (125, 2, 66, 90.0, 1531, True), (128, 1, 130, 200.0, 777, False), (160, 1, 36, 60.0, 1111, False),
           (200, 1, 70, 300.0, 640, True), (257, 2, 40, 120.0, 333, False)]
-# lengths of whole 16 samples: the plan's offset rows, from 33 channels on (64 * 2 coarse DMs: two full items)
-ROWS = [(33, 2, 20, 60.0, 16, False), (33, 1, 256, 40.0, 2512, True), (40, 2, 70, 900.0, 1008, False),
+# lengths of whole 16 samples and others (the tiling moved by 1 to 15), from 16 channels on (128 coarse DMs: two full items)
+ROWS = [(16, 3, 20, 60.0, 1003, True), (17, 2, 140, 90.0, 2001, False), (24, 2, 40, 300.0, 1, False),
+        (32, 2, 66, 60.0, 1538, True), (33, 2, 20, 60.0, 16, False), (33, 1, 256, 40.0, 2512, True),
+        (40, 2, 70, 900.0, 1008, False),
         (64, 2, 66, 90.0, 1536, True), (64, 1, 130, 200.0, 784, False), (64, 2, 40, 120.0, 779, False),
         (125, 2, 66, 90.0, 1536, False), (160, 1, 36, 60.0, 1120, True), (257, 1, 40, 120.0, 336, False)]
 
