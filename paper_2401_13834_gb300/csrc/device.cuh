@@ -110,6 +110,15 @@ __device__ __forceinline__ bool mbar_wait_or_abort(uint64_t* bar, uint32_t parit
   }
   return false;
 }
+// The same for a whole warp, which goes on or gives up together: lanes poll for
+// themselves, and one that saw the phase complete may stand beside one that ran out of
+// polls or saw the flag. A warp that issues copies and parted there would copy what its
+// lane 0 never announced, from places shuffled from lanes that have left. (The vote in
+// the consumers of k_stage1_wide costs 0.2% of a MeerKAT-L block.)
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, uint32_t polls,
+                                               const volatile int* abort) {
+  return __all_sync(0xffffffffu, mbar_wait_or_abort(bar, parity, polls, abort));
+}
 
 // ---------------------------------------------------------------------------
 // host side

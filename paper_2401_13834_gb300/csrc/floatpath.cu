@@ -301,7 +301,7 @@ __device__ __forceinline__ bool f1_consume(const F1Args& a, F1Shared& sh, const 
     for (int v = 0; v < VW; ++v) acc[i][v] = 0.f;
   for (int left = a.m; left > 0; left -= kF1Chan) {
     const int nc = min(left, kF1Chan);
-    if (!mbar_wait_or_abort(&sh.full[st], par, a.polls, &sh.abort_flag)) return false;
+    if (!mbar_wait_warp(&sh.full[st], par, a.polls, &sh.abort_flag)) return false;
     if (busy) {
       const float* r = stages + (size_t)st * kF1StageWords + j0;
       const uint2* t = reinterpret_cast<const uint2*>(stages + (size_t)st * kF1StageWords + kF1Chan * kF1RawWords) +
@@ -390,7 +390,7 @@ __global__ void __launch_bounds__(kF1Threads, 1) k_stage1_f32(const F1Args a) {
       const int cn = __shfl_sync(0xffffffffu, rec, 0), tw = __shfl_sync(0xffffffffu, rec, 1);
       const int to = __shfl_sync(0xffffffffu, rec, 2), dl = __shfl_sync(0xffffffffu, rec, 8 + (lane & 15));
       const int c0 = cn >> 5, nc = cn & 31;
-      if (q >= kF1Stages && !mbar_wait_or_abort(&sh.empty[st], par ^ 1u, a.polls, abort)) {
+      if (q >= kF1Stages && !mbar_wait_warp(&sh.empty[st], par ^ 1u, a.polls, abort)) {
         give_up();
         break;
       }

@@ -969,7 +969,7 @@ k_stage1_wide(const Src src, const int32_t* __restrict__ uoff, const int32_t* __
     bool end = false;
     while (true) {
       if (pw == 0) {
-        const bool ok = q < sp.nst || mbar_wait_or_abort(&sh.empty[st], par ^ 1u, polls, abort);
+        const bool ok = q < sp.nst || mbar_wait_warp(&sh.empty[st], par ^ 1u, polls, abort);
         if (!ok) give_up();
         if (lane == 0) {
           sh.item[st] = ok ? nextv : -1;
@@ -1039,7 +1039,7 @@ k_stage1_wide(const Src src, const int32_t* __restrict__ uoff, const int32_t* __
   if constexpr (!Src::kBatch) polls = src.get(0).polls; else polls = src.get(umem[0]).polls;
   int base = 0;   // rotates with the coarse DMs seen
   while (true) {
-    if (!mbar_wait_or_abort(&sh.full[st], par, polls, abort)) {
+    if (!mbar_wait_warp(&sh.full[st], par, polls, abort)) {
       give_up();
       return;
     }
@@ -1389,7 +1389,10 @@ k_stage2_u16(const Src src, const int32_t* __restrict__ uoff, const int32_t* __r
 // part[d][tile * SPLIT + (w % SPLIT)]. Every wait is bounded; a wait that
 // gives up raises a block-wide abort flag that every other wait sees, the
 // issuing warp waits (at the full limit) for the copies it has in flight, and
-// the block returns.
+// the block returns. The issuing warp goes on or gives up as a whole. Lanes of the
+// others decide for themselves: they copy nothing, and what a parted warp adds to the
+// sums is as invalid as the rest of the block's (a vote per chunk cost 1.5% of a
+// step of 64 small beams).
 constexpr int kPipeStages = kPipeStages2;
 constexpr int kPipeProc = kPipeProd2 - 1;   // processing warps (the other producer warp issues)
 
@@ -1509,7 +1512,7 @@ k_stage2_pipe(const Src src, const int32_t* __restrict__ uoff, const int32_t* __
       const int bq = (int)(q % kPipeStages);
       // the stage's previous chunk: every consumer has left it
       if (q >= kPipeStages &&
-          !mbar_wait_or_abort(&empty[bq], (uint32_t)((q / kPipeStages - 1) & 1), a.polls, abort)) {
+          !mbar_wait_warp(&empty[bq], (uint32_t)((q / kPipeStages - 1) & 1), a.polls, abort)) {
         give_up(a);
         break;
       }

@@ -131,7 +131,7 @@ k_stage2_pipe32(const Pipe32Args<E> a) {
       const int k = u / a.ntile;
       const int64_t t0 = (int64_t)(u - k * a.ntile) * tile_len;
       for (int ch = 0; ch < nchunk; ++ch, ++q) {
-        if (q >= a.nstage && !mbar_wait_or_abort(&empty[st], ph, a.polls, abort)) {
+        if (q >= a.nstage && !mbar_wait_warp(&empty[st], ph, a.polls, abort)) {
           give_up();
           go = false;
           break;
@@ -174,7 +174,7 @@ k_stage2_pipe32(const Pipe32Args<E> a) {
 #pragma unroll
       for (int v = 0; v < VW; ++v) acc[n][v] = (E)0;
     for (int ch = 0; ch < nchunk; ++ch) {
-      if (!mbar_wait_or_abort(&full[st], ph, a.polls, abort)) {
+      if (!mbar_wait_warp(&full[st], ph, a.polls, abort)) {
         give_up();
         return;
       }
