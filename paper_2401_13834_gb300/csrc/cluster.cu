@@ -348,17 +348,24 @@ __device__ __forceinline__ bool cl_near(const tx_clusterer& C, int dp, uint32_t 
   return __dadd_rn(__dmul_rn(gx, gx), __dmul_rn(gy, gy)) <= __dmul_rn(C.r, C.r);
 }
 
-// The times of row dq within r of point (d, t), as [lo, hi] (reach: the table's
-// entry for the two DMs).
-__device__ __forceinline__ void cl_interval(const tx_clusterer& C, int d, uint32_t t, int dq, int reach, uint32_t& lo,
-                                            uint32_t& hi) {
-  const uint32_t h = (uint32_t)(reach >> 1);
-  lo = t >= h ? t - h : 0u;
-  hi = t + h;
+// Calls f(lo, hi) for the times of row dq within r of point (d, t) (reach: the
+// table's entry for the two DMs), as intervals of the order of the keys, in which
+// negative times come last: one, or two where the times around t change sign. f
+// returns false to stop.
+template <typename F>
+__device__ __forceinline__ bool cl_interval(const tx_clusterer& C, int d, uint32_t tu, int dq, int reach, F&& f) {
+  const int t = (int)tu, h = reach >> 1;
+  int lo = t >= INT32_MIN + h ? t - h : INT32_MIN;
+  int hi = t <= INT32_MAX - h ? t + h : INT32_MAX;
   if (reach & 1) {
-    if (t >= h && !cl_near(C, d, t, dq, lo)) ++lo;   // an interval of none when h = 0
-    if (!cl_near(C, d, t, dq, hi)) hi = h ? hi - 1 : 0u;
+    const bool in_lo = t < INT32_MIN + h || cl_near(C, d, tu, dq, (uint32_t)lo);
+    const bool in_hi = t > INT32_MAX - h || cl_near(C, d, tu, dq, (uint32_t)hi);
+    if (h == 0 && !(in_lo && in_hi)) return true;   // none
+    lo += !in_lo;
+    hi -= !in_hi;
   }
+  if (hi >= 0 && !f((uint32_t)max(lo, 0), (uint32_t)hi)) return false;
+  return lo >= 0 || f((uint32_t)lo, (uint32_t)min(hi, -1));
 }
 
 // First entry of [b, e) whose time is at least t.
@@ -401,35 +408,38 @@ __global__ void k_cl_row_core(const tx_clusterer C, const unsigned long long* __
   const uint32_t t = (uint32_t)key[j];
   long long cnt = -1;   // the point itself is counted
   cl_rows(C, d, true, [&](int q, int reach) {
-    uint32_t lo, hi;
-    cl_interval(C, d, t, q, reach, lo, hi);
-    const int e = C.row[q + 1];
-    int p;
-    if (q == d) {   // up to k + 1 to the left of the point, then on to the right
-      p = j;
-      while (p > C.row[d] && (uint32_t)key[p - 1] >= lo && j - p <= C.k) --p;
-    } else {
-      p = cl_search(key, C.row[q], e, lo);
-    }
-    for (; p < e && (uint32_t)key[p] <= hi && cnt <= C.k; ++p) ++cnt;
-    return cnt <= C.k;
+    return cl_interval(C, d, t, q, reach, [&](uint32_t lo, uint32_t hi) {
+      const int e = C.row[q + 1];
+      int p;
+      if (q == d && lo <= t && t <= hi) {   // up to k + 1 to the left of the point, then on to the right
+        p = j;
+        while (p > C.row[d] && (uint32_t)key[p - 1] >= lo && j - p <= C.k) --p;
+      } else {
+        p = cl_search(key, C.row[q], e, lo);
+      }
+      for (; p < e && (uint32_t)key[p] <= hi && cnt <= C.k; ++p) ++cnt;
+      return cnt <= C.k;
+    });
   });
   C.core[j] = cnt > C.k;
 }
 
 // val[j] = j for the head of a run of core points, else 0: a core point whose
-// row's core point before it is out of reach.
+// row's core point before it is out of reach. Times of one sign make a run.
 __global__ void k_cl_row_heads(const tx_clusterer C, const unsigned long long* __restrict__ key, int n, int32_t* val) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= n) return;
   int v = 0;
   if (C.core[j]) {
     const int d = cl_dm(C, key[j]);
-    uint32_t lo, hi;
-    cl_interval(C, d, (uint32_t)key[j], d, __ldg(C.reach + (size_t)d * (C.nrow + 1)), lo, hi);
+    const uint32_t t = (uint32_t)key[j];
     v = j;
-    for (int p = j - 1; p >= C.row[d] && (uint32_t)key[p] >= lo; --p)
-      if (C.core[p]) { v = 0; break; }
+    cl_interval(C, d, t, d, __ldg(C.reach + (size_t)d * (C.nrow + 1)), [&](uint32_t lo, uint32_t hi) {
+      if (t < lo || t > hi) return true;
+      for (int p = j - 1; p >= C.row[d] && (uint32_t)key[p] >= lo; --p)
+        if (C.core[p]) { v = 0; break; }
+      return false;
+    });
   }
   val[j] = v;
 }
@@ -448,8 +458,8 @@ __device__ __forceinline__ void cl_cores(const tx_clusterer& C, const unsigned l
     while (p < e && (uint32_t)key[p] <= hi && !C.core[p]) ++p;
     if (p >= e || (uint32_t)key[p] > hi) return;
     f(p);
+    if (step >= hi - (uint32_t)key[p]) return;
     const uint32_t nt = (uint32_t)key[p] + step;   // the last time certainly in p's reach
-    if (nt >= hi) return;
     p = cl_search(key, p + 1, e, nt + 1);
   }
 }
@@ -460,11 +470,11 @@ __global__ void k_cl_row_union(const tx_clusterer C, const unsigned long long* _
   const int d = cl_dm(C, key[j]);
   const uint32_t t = (uint32_t)key[j];
   cl_rows(C, d, false, [&](int q, int reach) {   // each pair of rows once: later rows only
-    if (q == d) return true;
-    uint32_t lo, hi;
-    cl_interval(C, d, t, q, reach, lo, hi);
-    if (lo <= hi) cl_cores(C, key, q, lo, hi, [&](int p) { cl_unite(C.parent, j, p); });
-    return true;
+    if (q == d && ((int)t < 0 || (int)t > (reach >> 1))) return true;   // (of the own row: negative times from the others)
+    return cl_interval(C, d, t, q, reach, [&](uint32_t lo, uint32_t hi) {
+      if (q != d || (int)lo < 0) cl_cores(C, key, q, lo, hi, [&](int p) { cl_unite(C.parent, j, p); });
+      return true;
+    });
   });
 }
 
@@ -490,10 +500,10 @@ __global__ void k_cl_row_border(const tx_clusterer C, const unsigned long long* 
   const uint32_t t = (uint32_t)key[j];
   int best = INT32_MAX;
   cl_rows(C, d, true, [&](int q, int reach) {
-    uint32_t lo, hi;
-    cl_interval(C, d, t, q, reach, lo, hi);
-    if (lo <= hi) cl_cores(C, key, q, lo, hi, [&](int p) { best = min(best, C.label[p]); });
-    return true;
+    return cl_interval(C, d, t, q, reach, [&](uint32_t lo, uint32_t hi) {
+      cl_cores(C, key, q, lo, hi, [&](int p) { best = min(best, C.label[p]); });
+      return true;
+    });
   });
   C.label[j] = best == INT32_MAX ? -1 : best;
 }
