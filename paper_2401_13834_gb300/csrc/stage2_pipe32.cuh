@@ -25,53 +25,72 @@ struct Pipe32Args {
   uint32_t polls;
 };
 
-// Sums of D and D^2 over a warp's outputs. Integers are exact. Floats are
-// carried as (sum, compensation) pairs of float32 (TwoSum; the square as
-// TwoProduct), about 48 bits, and joined in double once per warp and unit: a
-// double add and multiply-add per output would cost 1.3 ms per 4096 x 65791
-// series at GB300's double rate, the pairs 0.1 ms.
-template <typename E>
-struct TileSums;
-template <>
-struct TileSums<int32_t> {
+// Sums of D and D^2 over a warp's outputs, VW of them per lane (0 where there is
+// none). Integers are exact. Floats: a lane's sum is carried as three float32 parts,
+// what one part's add rounds off going into the next, the square as TwoProduct. The
+// first two start at powers of two above any sum of the lane, so that an add's error
+// takes two operations more (Dekker's FastTwoSum) instead of five; they are taken off
+// again in double. The third's own rounding is below 2^-50 of the largest value, against
+// up to 2^-43 for adding 32 values in double: nothing is lost to the double sums. (Two
+// parts lose the second's rounding, up to 2^-43 of the sum, in the mean of equal values
+// a hundred times the error of double sums, which a variance far below the squared mean
+// magnifies.) A double add and multiply-add per output would cost 1.3 ms per 4096 x
+// 65791 series at GB300's double rate.
+template <int VW>
+__device__ __forceinline__ longlong2 tile_sums(const int32_t (&x)[VW]) {
   long long s1 = 0;
   unsigned long long s2 = 0;
-  __device__ __forceinline__ void add(int32_t v) {
-    s1 += v;
-    s2 += (unsigned long long)((long long)v * v);
-  }
-  __device__ __forceinline__ longlong2 warp_total() {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-      s2 += __shfl_xor_sync(0xffffffffu, s2, o);
-    }
-    return make_longlong2(s1, (long long)s2);
+  for (int v = 0; v < VW; ++v) {
+    s1 += x[v];
+    s2 += (unsigned long long)((long long)x[v] * x[v]);
   }
-};
-template <>
-struct TileSums<float> {
-  float s1 = 0.f, c1 = 0.f, s2 = 0.f, c2 = 0.f;
-  static __device__ __forceinline__ void comp(float& s, float& c, float x, float e) {
-    const float t = __fadd_rn(s, x), b = __fsub_rn(t, s);
-    c = __fadd_rn(c, __fadd_rn(__fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(x, b)), e));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    s1 += __shfl_xor_sync(0xffffffffu, s1, o);
+    s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+  }
+  return make_longlong2(s1, (long long)s2);
+}
+struct Sum3 {
+  float hi, mid, lo = 0.f;
+  float hi0, mid0;
+  // for up to 32 values below `top`, a power of two
+  __device__ __forceinline__ explicit Sum3(float top) : hi(64.f * top), mid(64.f * 64.f * 0x1p-24f * top), hi0(hi), mid0(mid) {}
+  static __device__ __forceinline__ float add_to(float& s, float x) {   // returns what the sum rounded off
+    const float t = __fadd_rn(s, x), e = __fsub_rn(x, __fsub_rn(t, s));
     s = t;
+    return e;
   }
-  __device__ __forceinline__ void add(float v) {
-    comp(s1, c1, v, 0.f);
-    const float p = __fmul_rn(v, v);
-    comp(s2, c2, p, __fmaf_rn(v, v, -p));
-  }
-  __device__ __forceinline__ double2 warp_total() {
-    double a = (double)s1 + (double)c1, b = (double)s2 + (double)c2;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      a += __shfl_xor_sync(0xffffffffu, a, o);
-      b += __shfl_xor_sync(0xffffffffu, b, o);
-    }
-    return make_double2(a, b);
+  __device__ __forceinline__ void add_mid(float x) { lo = __fadd_rn(lo, add_to(mid, x)); }
+  __device__ __forceinline__ void add(float x) { add_mid(add_to(hi, x)); }
+  __device__ __forceinline__ double total() const {
+    return ((double)hi - (double)hi0) + (((double)mid - (double)mid0) + (double)lo);
   }
 };
+template <int VW>
+__device__ __forceinline__ double2 tile_sums(const float (&x)[VW]) {
+  static_assert(VW <= 32, "Sum3 holds the sum of 32 values");
+  float most = 0.f;
+#pragma unroll
+  for (int v = 0; v < VW; ++v) most = fmaxf(most, fabsf(x[v]));
+  const float top = __uint_as_float((__float_as_uint(most) & 0x7F800000u) + 0x00800000u);   // the power of two above
+  Sum3 s1(top), s2(top * top);
+#pragma unroll
+  for (int v = 0; v < VW; ++v) {
+    s1.add(x[v]);
+    const float p = __fmul_rn(x[v], x[v]);
+    s2.add(p);
+    s2.add_mid(__fmaf_rn(x[v], x[v], -p));
+  }
+  double a = s1.total(), b = s2.total();
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    b += __shfl_xor_sync(0xffffffffu, b, o);
+  }
+  return make_double2(a, b);
+}
 
 // Persistent blocks walk units (coarse group k, tile of 32 VW split outputs)
 // in sub-band chunks through `nstage` shared-memory stages. The last warp
@@ -207,14 +226,13 @@ k_stage2_pipe32(const Pipe32Args<E> a) {
       if (g + 16 * n >= nd) continue;
       const int d = dfirst + g + 16 * n;
       E* drow = a.D + (size_t)d * a.Dp;
-      TileSums<E> sum;
 #pragma unroll
       for (int v = 0; v < VW; ++v) {
         const int64_t t = t0 + 32 * v;
         if (t < a.Td) drow[t] = acc[n][v];
-        if (t < a.T) sum.add(acc[n][v]);
+        if (t >= a.T) acc[n][v] = (E)0;
       }
-      const auto tot = sum.warp_total();
+      const auto tot = tile_sums(acc[n]);
       if (lane == 0)
         reinterpret_cast<std::remove_const_t<decltype(tot)>*>(a.part)[((size_t)d * a.ntile + tile) * a.split + part_i] =
             tot;
