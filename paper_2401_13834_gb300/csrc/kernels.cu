@@ -773,12 +773,11 @@ int32_t tx_downsample(const uint8_t* d_in, int32_t layout, int32_t nchan, int64_
 // below, which every GPU that loads this library holds until the process exits.
 namespace {
 
-constexpr size_t kNoAllocScratchBytes = size_t(32) << 20;  // 32 MiB per device
 constexpr int kNoAllocMaxDevices = 64;
 
 }  // namespace
 
-static __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocScratchBytes];
+static __device__ __align__(256) uint8_t g_noalloc_scratch[kNoAllocScratchBytes];   // per device
 
 namespace {
 
@@ -833,9 +832,9 @@ int32_t tx_dedisperse_noalloc(const tx_plan* p, const uint8_t* d_x, int64_t ld, 
   const size_t b_tab2 = align256(p->tab2.size() * 4);
   const size_t b_ctr = 256;   // the stage-1 item counter
   const size_t need = b_items + b_d1 + b_abase + b_e2 + b_P + b_part + b_tab2 + b_ctr;
-  if (need > kNoAllocScratchBytes) {
-    set_error("this plan needs %zu bytes of scratch; the static scratch of tx_dedisperse_noalloc holds %zu",
-              need, kNoAllocScratchBytes);
+  if (need > (size_t)kNoAllocScratchBytes) {
+    set_error("this plan needs at least %zu bytes of scratch; the static scratch of tx_dedisperse_noalloc holds %zu",
+              need, (size_t)kNoAllocScratchBytes);
     return TX_ERR_BUDGET;
   }
   void* scratch = nullptr;

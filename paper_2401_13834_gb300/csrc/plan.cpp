@@ -67,32 +67,32 @@ Wide1Shape wide1_shape(int m, int most) {
   return r;
 }
 
-// Appends the offset rows of the wide stage 1 for sub-band s, coarse DMs [kb, ke)
-// to tab1, for windows that start with tab1_phase: s1w.tsu words each, {channels
+// Writes the offset rows of the wide stage 1 for sub-band s, coarse DMs [kb, ke)
+// from `row` on, for windows that start with tab1_phase: s1w.tsu words each, {channels
 // of residue 3 | residue 2 << 16, residue 1 | residue 0 << 16}, two unused, then
 // the channels' byte offsets (of words) residue by residue, each part but the
 // last padded to four. Rows sorted by the producer warps instead took the kernel
 // from 2.49 to 2.73 ms on the MeerKAT-L block; there the rows are 5 MB.
-static void wide1_table(tx_plan* p, int s, int kb, int ke) {
-  const int m = p->m, tsu = p->s1w.tsu;
+static void wide1_table(const tx_plan* p, int s, int kb, int ke, int32_t* row) {
+  const int m = p->m, rb = p->s1w.rb;   // rb is a multiple of 16
   const int32_t* d0 = p->d1.data() + (size_t)kb * p->nchan + (size_t)s * m;
-  for (int k = kb; k < ke; ++k) {
+  int32_t pre[257];   // a channel's offset less its delay
+  for (int c = 0; c < m; ++c) pre[c] = c * rb + ((p->tab1_phase + d0[c]) & 15) - d0[c];
+  for (int k = kb; k < ke; ++k, row += p->s1w.tsu) {
     const int32_t* dk = p->d1.data() + (size_t)k * p->nchan + (size_t)s * m;
-    const size_t at = p->tab1.size();
-    p->tab1.resize(at + tsu, 0);
-    int32_t* row = p->tab1.data() + at;
-    int pos = 4, cnt[4] = {0, 0, 0, 0};
+    uint64_t n = 0;   // channels of residue r in bits 16 r ..
+    for (int c = 0; c < m; ++c) n += 1ull << (16 * ((pre[c] + dk[c]) & 3));
+    row[0] = (int32_t)(n >> 48 | (n >> 32 & 0xFFFF) << 16);
+    row[1] = (int32_t)((n >> 16 & 0xFFFF) | (n & 0xFFFF) << 16);
+    int pos[4], at = 4;
     for (int r = 3; r >= 0; --r) {
-      pos = (pos + 3) & ~3;
-      for (int c = 0; c < m; ++c) {
-        const int32_t x = ((p->tab1_phase + d0[c]) & 15) + dk[c] - d0[c];
-        if ((x & 3) != r) continue;
-        row[pos++] = c * p->s1w.rb + (x & ~3);
-        ++cnt[r];
-      }
+      pos[r] = at;
+      at += (int)((n >> (16 * r) & 0xFFFF) + 3) & ~3;
     }
-    row[0] = cnt[3] | cnt[2] << 16;
-    row[1] = cnt[1] | cnt[0] << 16;
+    for (int c = 0; c < m; ++c) {
+      const int32_t x = pre[c] + dk[c];
+      row[pos[x & 3]++] = x & ~3;
+    }
   }
 }
 
@@ -168,15 +168,24 @@ static int32_t float_chunks(tx_plan* p, int s, int kb, int ke) {
   return nchunk;
 }
 
-// The work items of the integer stage 1: the wide kernel's in its shape s1w or
-// k_stage1's, with their offset tables in tab1 where `tab` is set.
-static void stage1_items(tx_plan* p, bool wide, bool tab, std::vector<Stage1Item>& items) {
+// The work of the integer stage 1 by sub-band and coarse DMs: the wide kernel's in
+// its shape s1w, or k_stage1's; tile step, range of tiles, words of the offset
+// tables and number of items of them all.
+struct Stage1Groups {
+  struct Group {   // the items of (s, [kb, ke)), at times from first * step on
+    Stage1Item it;
+    int64_t first, count;
+  };
+  std::vector<Group> groups;
+  int64_t step = 1, t_lo = INT64_MAX, t_hi = INT64_MIN, words = 0, items = 0;
+};
+
+static Stage1Groups stage1_groups(const tx_plan* p, bool wide) {
   const int m = p->m, nk = p->nk, nsub = p->nsub, nchan = p->nchan, q1 = p->q1;
   const int span_max = wide ? p->s1w.span : q1 - 16, most = wide ? p->s1w.nmax : kStage1MaxCoarse;
-  const int64_t step = wide ? kWide1TileStep(p->s1w.vw) : 4 * (int64_t)q1;
-  const int TS1 = (m + 3) & ~3, SW1 = kStage1StagedWords(q1);
-  items.clear();
-  if (tab) p->tab1.clear();
+  const int TS1 = (m + 3) & ~3;
+  Stage1Groups r;
+  r.step = wide ? kWide1TileStep(p->s1w.vw) : 4 * (int64_t)q1;
   for (int s = 0; s < nsub; ++s) {
     int kb = 0;
     while (kb < nk) {
@@ -199,29 +208,53 @@ static void stage1_items(tx_plan* p, bool wide, bool tab, std::vector<Stage1Item
         hi = std::max<int64_t>(hi, (int64_t)p->abase[(size_t)k * nsub + s] + p->Pp);
       }
       if (wide) hi += 12;   // (a multiple of 4 below 16: see wide1_early)
-      const int32_t toff = tab ? (int32_t)p->tab1.size() : 0;
-      if (tab && wide) {
-        wide1_table(p, s, kb, ke);
-      } else if (tab) {
-        for (int kk = 0; kk < ke - kb; ++kk)
-          for (int c = 0; c < TS1; ++c) {
-            if (c >= m) { p->tab1.push_back(0); continue; }
-            const int32_t d0 = p->d1[(size_t)kb * nchan + s * m + c];
-            p->tab1.push_back(c * SW1 + ((p->tab1_phase + d0) & 15) + p->d1[(size_t)(kb + kk) * nchan + s * m + c] - d0);
-          }
-        for (int kk = 0; kk < ((ke - kb + 3) & ~3); ++kk)   // the coarse DMs' P-row bases
-          p->tab1.push_back(kk < ke - kb ? p->abase[(size_t)(kb + kk) * nsub + s] : 0);
-      }
-      for (int64_t t0 = floor_div(lo, step) * step; t0 < hi; t0 += step)
-        items.push_back(Stage1Item{s, kb, ke, (int32_t)t0, span, toff, 0, 0});
+      const int64_t first = floor_div(lo, r.step), last = floor_div(hi - 1, r.step);
+      r.groups.push_back({Stage1Item{s, kb, ke, 0, span, (int32_t)r.words, 0, 0}, first, last - first + 1});
+      r.t_lo = std::min(r.t_lo, first);
+      r.t_hi = std::max(r.t_hi, last);
+      r.words += wide ? (int64_t)(ke - kb) * p->s1w.tsu : (int64_t)(ke - kb) * TS1 + ((ke - kb + 3) & ~3);
+      r.items += last - first + 1;
       kb = ke;
     }
   }
-  // Time-major order: blocks working at the same time read overlapping input
-  // windows of every sub-band, which keeps the ring's working set in L2.
-  std::stable_sort(items.begin(), items.end(), [](const Stage1Item& a, const Stage1Item& b) {
-    return a.tau0 != b.tau0 ? a.tau0 < b.tau0 : (a.s != b.s ? a.s < b.s : a.kb < b.kb);
-  });
+  return r;
+}
+
+// Their items in order of time, then sub-band and coarse DMs: blocks working at the
+// same time read overlapping input windows of every sub-band, which keeps the
+// ring's working set in L2.
+static void stage1_items(const Stage1Groups& r, std::vector<Stage1Item>& items) {
+  std::vector<int64_t> at((size_t)(r.t_hi - r.t_lo + 2), 0);   // items before each time
+  for (const auto& g : r.groups)
+    for (int64_t i = 0; i < g.count; ++i) ++at[(size_t)(g.first - r.t_lo + i + 1)];
+  for (size_t i = 1; i < at.size(); ++i) at[i] += at[i - 1];
+  items.resize((size_t)r.items);
+  for (const auto& g : r.groups)
+    for (int64_t i = 0; i < g.count; ++i) {
+      Stage1Item it = g.it;
+      it.tau0 = (int32_t)((g.first + i) * r.step);
+      items[(size_t)at[(size_t)(g.first - r.t_lo + i)]++] = it;
+    }
+}
+
+// Their offset tables, into tab1.
+static void stage1_tables(tx_plan* p, bool wide, const Stage1Groups& r) {
+  const int m = p->m, nchan = p->nchan, TS1 = (m + 3) & ~3, SW1 = kStage1StagedWords(p->q1);
+  p->tab1.assign((size_t)r.words, 0);
+  for (const auto& g : r.groups) {
+    const int s = g.it.s, kb = g.it.kb, ke = g.it.ke;
+    int32_t* t = p->tab1.data() + g.it.tab;
+    if (wide) {
+      wide1_table(p, s, kb, ke, t);
+      continue;
+    }
+    const int32_t* d0 = p->d1.data() + (size_t)kb * nchan + (size_t)s * m;
+    for (int k = kb; k < ke; ++k, t += TS1) {
+      const int32_t* dk = p->d1.data() + (size_t)k * nchan + (size_t)s * m;
+      for (int c = 0; c < m; ++c) t[c] = c * SW1 + ((p->tab1_phase + d0[c]) & 15) + dk[c] - d0[c];
+    }
+    for (int k = kb; k < ke; ++k) *t++ = p->abase[(size_t)k * p->nsub + s];   // the coarse DMs' P-row bases
+  }
 }
 
 static int build(tx_plan* p, const tx_plan_desc* d) {
@@ -472,16 +505,22 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
   // every window start of an execute is (head - L) mod R with head a multiple
   // of 64 plus a multiple of T, and R a multiple of 64
   p->tab1_phase = (int32_t)((16 - p->L % 16) % 16);
-  while (p->interm != TX_INTERM_F32) {   // (the float path has its own list)
-    stage1_items(p, p->wide1 != 0, true, p->items1);
+  if (p->interm != TX_INTERM_F32) {   // (the float path has its own list)
+    Stage1Groups work = stage1_groups(p, p->wide1 != 0);
     // few items: shorter tiles of the wide kernel keep the SMs busy
-    const Wide1Shape next = wide1_shape(m, p->s1w.vw / 2);
-    if (!p->wide1 || p->items1.size() >= (size_t)kWide1MinItems || p->s1w.vw <= 2 || next.nst < 2) break;
-    p->s1w = next;
+    while (p->wide1 && work.items < kWide1MinItems && p->s1w.vw > 2) {
+      const Wide1Shape next = wide1_shape(m, p->s1w.vw / 2);
+      if (next.nst < 2) break;
+      p->s1w = next;
+      work = stage1_groups(p, true);
+    }
+    stage1_items(work, p->items1);
+    stage1_tables(p, p->wide1 != 0, work);
   }
   // tx_dedisperse_noalloc runs k_stage1 in any case: its static scratch has no room for the rows
-  if (p->interm == TX_INTERM_U16) {
-    if (p->wide1) stage1_items(p, false, false, p->items_na);
+  // (nor for plans whose stage-1 sums alone fill it)
+  if (p->interm == TX_INTERM_U16 && (int64_t)nk * nsub * p->Pp * 2 <= kNoAllocScratchBytes) {
+    if (p->wide1) stage1_items(stage1_groups(p, false), p->items_na);
     else p->items_na = p->items1;
   }
   if (p->interm == TX_INTERM_F32) {

@@ -36,6 +36,7 @@ constexpr int kWide1Producers = 4;     // copying warps
 constexpr int kWide1Warps = kWide1Consumers + kWide1Producers;
 constexpr int kWide1MaxStages = 8;     // items in flight
 constexpr int kWide1TileStep(int vw) { return 128 * vw - 16; }
+constexpr int64_t kNoAllocScratchBytes = 32 << 20;   // static device scratch of tx_dedisperse_noalloc
 constexpr int kSmemMax = 232448;       // opt-in dynamic shared memory per block (227 KB)
 
 // Polls of an mbarrier before a kernel gives up waiting for a bulk copy; each
@@ -205,7 +206,7 @@ struct tx_plan {
   std::vector<uint32_t> tab_f;
   int32_t phases_f = 1, phase0_f = 0;
   std::vector<tx::Stage1Item> items1;
-  std::vector<tx::Stage1Item> items_na;   // tx_dedisperse_noalloc's, for k_stage1
+  std::vector<tx::Stage1Item> items_na;   // tx_dedisperse_noalloc's, for k_stage1 (none where its scratch cannot hold the sums)
   // stage-1 offset tables, per (s, kb, ke): rows kk < ke - kb of (m + 3) & ~3
   // words, word c = c * staged words + ((tab1_phase + d1[kb][c]) & 15) +
   // d1[kb + kk][c] - d1[kb][c], then abase[kb + kk][s] for kk < ke - kb

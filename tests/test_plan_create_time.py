@@ -1,0 +1,26 @@
+"""Creating a plan whose stage 1 runs the wide sub-bands' kernel costs little more
+than one of the same shape that does not (a shorter tile asked for): its work list and
+tables are built once. CPU time of the fastest of interleaved runs; a slow plan is
+slow in every round, so one quick round is enough."""
+import time
+
+import synth
+
+
+def _ratio(tx, wl, interm):
+    best = [1e9, 1e9]
+    for _ in range(25):
+        for i, q in enumerate((0, 128)):
+            t = time.process_time()
+            tx.Plan(wl.freqs_mhz, wl.tsamp_s, wl.dms, wl.nsub, wl.widths, wl.nsamp, group=wl.group, interm=interm,
+                    tile_q1=q)
+            best[i] = min(best[i], time.process_time() - t)
+    return best[0] / best[1]
+
+
+def test_wide_plans_cost_little_more():
+    import paper_2401_13834_gb300 as tx
+    # 64 channels per sub-band, few items: three lengths of tile are tried
+    wl = synth.tiny_workload(nchan=512, nsub=8, ndm=512, nsamp=8000, dm_max=200.0, widths=(1, 2, 4), tsamp=100e-6, group=2)
+    for interm in ("u16", "i32"):
+        assert any(_ratio(tx, wl, interm) < 1.6 for _ in range(4)), interm
