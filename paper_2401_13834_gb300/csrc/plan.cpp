@@ -502,6 +502,8 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
   // residues leave little between shifts: below 16 k_stage1 stays.
   p->s1w = wide1_shape(m, 8);
   p->wide1 = p->s1w.nst >= 2 && (q1 < 256 ? stage1_smem_bytes(m, 2 * q1) > kSmemMax : m >= 16);
+  // (an item's place in the tables is 32 bits; the wide kernel's rows are up to twice k_stage1's)
+  if ((int64_t)nk * nsub * p->s1w.tsu > INT32_MAX) p->wide1 = 0;
   // every window start of an execute is (head - L) mod R with head a multiple
   // of 64 plus a multiple of T, and R a multiple of 64
   p->tab1_phase = (int32_t)((16 - p->L % 16) % 16);
