@@ -138,8 +138,11 @@ typedef struct tx_plan_desc {
                                     outputs) or 2, 4, 8 (tiles of 1024), with
                                     min(group, 32) * tile_split2 <= 32; 0 = 8, 4, 2
                                     or 1 for groups of <= 4, 8, 16 or more; used by
-                                    groups of more than 16 DMs (smaller groups run
-                                    the pipelined stage 2, which sizes itself)   */
+                                    16-bit intermediates with groups of more than
+                                    16 DMs (smaller groups and 32-bit intermediates
+                                    run pipelined stage 2s that size themselves; for
+                                    the latter it only bounds the delay spread of a
+                                    group that is taken, by a row of such a tile) */
   int32_t        norm;           /* enum tx_norm; TX_NORM_NONE unless interm is
                                     TX_INTERM_F32, which needs another mode. The
                                     float path runs single beams (tx_execute,
@@ -166,7 +169,9 @@ typedef struct tx_plan_info {
                                a block that wraps its end is ingested in two launches */
   int64_t ring_head0;       /* where a fresh beam's first block lands in it        */
   int32_t tile_q1;          /* the stage-1 tile chosen (see tx_plan_desc)           */
-  int32_t tile_split2;      /* the stage-2 warps per fine DM chosen                 */
+  int32_t tile_split2;      /* the stage-2 warps per fine DM chosen (32-bit
+                               intermediates: tx_plan_desc's value as resolved,
+                               which their stage 2 does not use)                 */
   int64_t workspace_bytes_compact;   /* d_workspace of an execute on a compact beam */
   int64_t compact_beam_state_bytes;  /* device memory one compact beam holds        */
 } tx_plan_info;

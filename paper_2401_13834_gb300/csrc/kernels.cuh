@@ -140,8 +140,9 @@ __device__ __forceinline__ void madd_hi16(uint32_t& acc, uint32_t a) {
 
 // lo += the low half of w, hi += its high half, in FP32: one mixed-precision add
 // each instead of a conversion and an add (MeerKAT-L stage 2 from FP16: 1.79 ->
-// 1.38 ms, the uint16 form's time). The halves hold integers and the sums stay
-// below 2^24, so every add is exact.
+// 1.38 ms, the uint16 form's time). The halves hold integers of at most 255 times
+// their sub-band's channels in size, so up to 65793 channels every sum stays
+// below 2^24 and every add is exact.
 __device__ __forceinline__ void add_halves(float& lo, float& hi, uint32_t w) {
   asm("{\n\t.reg .f16 l, h;\n\tmov.b32 {l, h}, %2;\n\tadd.f32.f16 %0, l, %0;\n\tadd.f32.f16 %1, h, %1;\n\t}"
       : "+f"(lo), "+f"(hi)
@@ -813,7 +814,7 @@ k_stage1(const Src src, const int32_t* __restrict__ uoff, const int32_t* __restr
 // stage 1 of wide sub-bands
 // ---------------------------------------------------------------------------
 // Adds `cnt` channels' words to the sums: aw the words themselves, ah their odd
-// bytes as 16-bit lanes. e: the channels' byte offsets (16-byte aligned).
+// bytes as 16-bit lanes. e: the channels' byte offsets, from a 16-byte aligned address.
 template <int VW>
 __device__ __forceinline__ void wide1_add(uint32_t (&aw)[VW], uint32_t (&ah)[VW], const uint8_t* __restrict__ base,
                                            const uint32_t* __restrict__ e, int cnt, uint32_t one) {
@@ -1326,7 +1327,7 @@ k_stage2_u16(const Src src, const int32_t* __restrict__ uoff, const int32_t* __r
         const int64_t ta = t0 + 2 * (jbase + lane + 32 * v);
         uint32_t lo, hi;
         if constexpr (HALF) {
-          // the halves hold integers and their FP32 sums stay below 2^24: exact
+          // integers: their FP32 sums are exact (see add_halves)
           lo = (uint32_t)((int)fl[v] + O);
           hi = (uint32_t)((int)fh[v] + O);
         } else {
@@ -1665,7 +1666,7 @@ k_stage2_pipe(const Src src, const int32_t* __restrict__ uoff, const int32_t* __
             const int64_t ta = cc.t0 + 2 * (jbase + lane + 32 * v);
             uint32_t lo, hi;
             if constexpr (HALF) {
-              // the halves hold integers and their FP32 sums stay below 2^24: exact
+              // integers: their FP32 sums are exact (see add_halves)
               lo = (uint32_t)((int)fl[v] + O);
               hi = (uint32_t)((int)fh[v] + O);
             } else {

@@ -131,8 +131,8 @@ static int auto_group(const std::vector<double>& f, double tsamp, int nsub, int 
 }
 
 // Float path stage 1: outputs per lane of a warp for n coarse DMs. A warp sums
-// four consecutive coarse DMs over the tile (16 outputs per lane), or a half,
-// quarter or eighth of it where fewer coarse DMs would leave warps idle.
+// four consecutive coarse DMs over half the tile (8 outputs per lane), or a quarter
+// or an eighth of it where fewer coarse DMs would leave warps idle.
 static int32_t float_outputs(int n) {
   const int quads = (n + kF1Quad - 1) / kF1Quad;
   int vw = kF1Outputs;
@@ -423,8 +423,8 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
   p->ntile2 = (int32_t)((p->Td + tt2 - 1) / tt2);
   p->sww2 = (int32_t)round_up(p->nw2 + (span2 + 7 + 2) / 2 + 6, 4);
   const int64_t last_t0 = (int64_t)(p->ntile2 - 1) * tt2;
-  // uint16 path reads [base, base + 2 sww2) with base <= t0 + 15; int32 path
-  // reads [t0 + emin, + tt2 + span2 + 16)
+  // 16-bit stage 2 reads [base, base + 2 sww2) with base <= t0 + 15, the 32-bit
+  // one [t0 + 8, + sw32) at most, sw32 <= tt2 + span2 + 11
   p->Pp = round_up(std::max<int64_t>(last_t0 + 16 + 2 * (int64_t)p->sww2, last_t0 + 16 + tt2 + span2 + 16) + 16, 64);
   if (p->pipe2) {
     // per stage: even and odd slots of sww2 words per sub-band, and the address table
@@ -495,11 +495,12 @@ static int build(tx_plan* p, const tx_plan_desc* d) {
   if (stage1_smem_bytes(m, q1) > kSmemMax) { set_error("too many channels per sub-band for stage 1 (%d)", m); return TX_ERR_UNSUPPORTED; }
   p->q1 = q1;
   // The wide kernel, unless a tile shorter than the longest that fits is asked
-  // for. Stage 1 of k_stage1 and of it: 16 channels per sub-band 1.06 and 0.91 ms
-  // (1024 channels, 4096 DMs, 65536 samples), 32 channels 1.62 and 1.49, 64
-  // channels 2.70 and 2.49 (4096 channels), 125 channels 231 and 82 us (where
-  // k_stage1's tiles shrink to 256 samples). Few channels spread over the four
-  // residues leave little between shifts: below 16 k_stage1 stays.
+  // for. Stage 1 of k_stage1 and of it: 16 channels per sub-band 1.06 and 0.92 ms
+  // (64 sub-bands, 4096 DMs, 65536 samples), 32 channels 1.62 and 1.49, 64
+  // channels 2.70 and 2.50, 125 channels 231 and 82 us (1000 channels; k_stage1's
+  // tiles shrink to 256 samples). The two do not meet at 16: 12 channels take 0.92 and
+  // 0.78 ms, 8 channels 0.79 and 0.65 (16 sub-bands, 128 DMs, 16384 samples:
+  // 15.3 and 12.4 us), so the line could lie lower.
   p->s1w = wide1_shape(m, 8);
   p->wide1 = p->s1w.nst >= 2 && (q1 < 256 ? stage1_smem_bytes(m, 2 * q1) > kSmemMax : m >= 16);
   // (an item's place in the tables is 32 bits; the wide kernel's rows are up to twice k_stage1's)
