@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(kThreads) k_norm_ingest_tf(const uint8_t* __re
 // make a warp's part 256 outputs, 8 independent loads in flight per coarse DM,
 // for up to 40 coarse DMs on 20 warps.
 // One block per item that staged all its channels, then summed, took 12.57
-// ms on that block; this takes 7.63 ms with shared memory and issue both 80%
+// ms on that block; this takes 7.59 ms with shared memory and issue both 80%
 // busy (every load taken: 8.30; 30 warps, which spill: 12.5; predicated loads
 // instead of branches, which keep their shared-memory slots: 8.25). Waits are
 // bounded as in k_stage2_pipe.

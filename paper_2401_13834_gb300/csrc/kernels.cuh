@@ -922,9 +922,9 @@ struct Wide1Shared {
 // windows into 32-bit words four times their size; here they stay bytes, which
 // leaves room for a second item in flight and, past 64 channels, for tiles of
 // 512 outputs and 64 coarse DMs where k_stage1's shrink. Measured, k_stage1 and
-// this: MeerKAT-L block 2.70 and 2.49 ms; 1024 channels of 64 per sub-band, 1024
-// DMs, 32768 samples 403 and 350 us (32771 samples 419 and 360); 125 channels per
-// sub-band (1000 channels, 76 coarse DMs, 20160 samples) 231 and 82 us.
+// this: MeerKAT-L block 2.70 and 2.50 ms; 1024 channels of 64 per sub-band, 1024
+// DMs, 32768 samples 403 and 352 us (32771 samples 419 and 364); 125 channels per
+// sub-band (1000 channels, 76 coarse DMs, 20160 samples) 231 and 83 us.
 // Waits are bounded as in k_stage2_pipe; only one producer warp waits for free
 // stages, the others follow it through a named barrier.
 template <int VW, typename PT, typename Src, bool HALF = false>

@@ -106,7 +106,7 @@ __device__ __forceinline__ double2 tile_sums(const float (&x)[VW]) {
 // spread (up to about 440 samples on MeerKAT-L) a small part of what is
 // staged, and 16 to 28 consumer warps of 8 to 32 independent sums keep the
 // loads in flight. 4096 DMs x 64 sub-bands x 65791 outputs: float32 3.90 ->
-// 2.03 ms, int32 11.99 -> 1.93 ms against one block per tile that staged its
+// 2.02 ms, int32 11.99 -> 1.94 ms against one block per tile that staged its
 // rows with 4-byte copies between block-wide barriers. Waits are bounded as
 // in k_stage2_pipe.
 template <typename E, int VW, int NDM>
