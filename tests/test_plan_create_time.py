@@ -19,6 +19,8 @@ def _ratio(tx, wl, interm):
 
 
 def test_wide_plans_cost_little_more():
+    from paper_2401_13834_gb300 import build
+    build.build()
     import paper_2401_13834_gb300 as tx
     # 64 channels per sub-band, few items: three lengths of tile are tried
     wl = synth.tiny_workload(nchan=512, nsub=8, ndm=512, nsamp=8000, dm_max=200.0, widths=(1, 2, 4), tsamp=100e-6, group=2)
