@@ -350,10 +350,11 @@ __device__ __forceinline__ bool cl_near(const tx_clusterer& C, int dp, uint32_t 
 
 // Calls f(lo, hi) for the times of row dq within r of point (d, t) (reach: the
 // table's entry for the two DMs), as intervals of the order of the keys, in which
-// negative times come last: one, or two where the times around t change sign. f
-// returns false to stop.
+// negative times come last: one, or two where the times around t change sign. The
+// row is not empty. f returns false to stop.
 template <typename F>
-__device__ __forceinline__ bool cl_interval(const tx_clusterer& C, int d, uint32_t tu, int dq, int reach, F&& f) {
+__device__ __forceinline__ bool cl_interval(const tx_clusterer& C, const unsigned long long* __restrict__ key, int d,
+                                            uint32_t tu, int dq, int reach, F&& f) {
   const int t = (int)tu, h = reach >> 1;
   int lo = t >= INT32_MIN + h ? t - h : INT32_MIN;
   int hi = t <= INT32_MAX - h ? t + h : INT32_MAX;
@@ -364,8 +365,14 @@ __device__ __forceinline__ bool cl_interval(const tx_clusterer& C, int d, uint32
     lo += !in_lo;
     hi -= !in_hi;
   }
-  if (hi >= 0 && !f((uint32_t)max(lo, 0), (uint32_t)hi)) return false;
-  return lo >= 0 || f((uint32_t)lo, (uint32_t)min(hi, -1));
+  uint32_t a = (uint32_t)(hi >= 0 ? max(lo, 0) : lo), b = (uint32_t)hi;
+#pragma unroll 1   // f once in the code
+  while (f(a, b)) {
+    if (lo >= 0 || a == (uint32_t)lo || (int)(uint32_t)key[C.row[dq + 1] - 1] >= 0) return true;   // (none negative)
+    a = (uint32_t)lo;
+    b = 0xFFFFFFFFu;
+  }
+  return false;
 }
 
 // First entry of [b, e) whose time is at least t.
@@ -408,7 +415,7 @@ __global__ void k_cl_row_core(const tx_clusterer C, const unsigned long long* __
   const uint32_t t = (uint32_t)key[j];
   long long cnt = -1;   // the point itself is counted
   cl_rows(C, d, true, [&](int q, int reach) {
-    return cl_interval(C, d, t, q, reach, [&](uint32_t lo, uint32_t hi) {
+    return cl_interval(C, key, d, t, q, reach, [&](uint32_t lo, uint32_t hi) {
       const int e = C.row[q + 1];
       int p;
       if (q == d && lo <= t && t <= hi) {   // up to k + 1 to the left of the point, then on to the right
@@ -434,7 +441,7 @@ __global__ void k_cl_row_heads(const tx_clusterer C, const unsigned long long* _
     const int d = cl_dm(C, key[j]);
     const uint32_t t = (uint32_t)key[j];
     v = j;
-    cl_interval(C, d, t, d, __ldg(C.reach + (size_t)d * (C.nrow + 1)), [&](uint32_t lo, uint32_t hi) {
+    cl_interval(C, key, d, t, d, __ldg(C.reach + (size_t)d * (C.nrow + 1)), [&](uint32_t lo, uint32_t hi) {
       if (t < lo || t > hi) return true;
       for (int p = j - 1; p >= C.row[d] && (uint32_t)key[p] >= lo; --p)
         if (C.core[p]) { v = 0; break; }
@@ -471,7 +478,7 @@ __global__ void k_cl_row_union(const tx_clusterer C, const unsigned long long* _
   const uint32_t t = (uint32_t)key[j];
   cl_rows(C, d, false, [&](int q, int reach) {   // each pair of rows once: later rows only
     if (q == d && ((int)t < 0 || (int)t > (reach >> 1))) return true;   // (of the own row: negative times from the others)
-    return cl_interval(C, d, t, q, reach, [&](uint32_t lo, uint32_t hi) {
+    return cl_interval(C, key, d, t, q, reach, [&](uint32_t lo, uint32_t hi) {
       if (q != d || (int)lo < 0) cl_cores(C, key, q, lo, hi, [&](int p) { cl_unite(C.parent, j, p); });
       return true;
     });
@@ -500,7 +507,7 @@ __global__ void k_cl_row_border(const tx_clusterer C, const unsigned long long* 
   const uint32_t t = (uint32_t)key[j];
   int best = INT32_MAX;
   cl_rows(C, d, true, [&](int q, int reach) {
-    return cl_interval(C, d, t, q, reach, [&](uint32_t lo, uint32_t hi) {
+    return cl_interval(C, key, d, t, q, reach, [&](uint32_t lo, uint32_t hi) {
       cl_cores(C, key, q, lo, hi, [&](int p) { best = min(best, C.label[p]); });
       return true;
     });
